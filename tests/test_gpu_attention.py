@@ -739,3 +739,24 @@ def test_l2_prefetch_depth_changes_no_result(cuda_device, tiles):
         cmc.set_l2_prefetch_tiles(5)
     for a, b in zip(outs[5], outs[tiles]):
         np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("L,Hkv,d", [(1, 1, 64), (1, 128, 64), (1, 129, 64), (3, 43, 128),
+                                     (16, 16, 128), (33, 16, 128), (80, 8, 128)])
+def test_window_append_one_cta_and_clusters(cuda_device, L, Hkv, d):
+    """One CTA per sequence up to 2,048 chunks of 16 bytes, then clusters of 2, 4 and 8, the last
+    with more than one round of chunks a thread; a position past 2^32 and an invalid one."""
+    W, pos0 = 7, [0, 6, 7, (1 << 32) + 5, -1]
+    g = torch.Generator().manual_seed(L * Hkv)
+    shape = (len(pos0), L, Hkv, W, d)
+    ring = [torch.randn(shape, generator=g).to(torch.bfloat16) for _ in range(2)]
+    new = [torch.randn(shape[:3] + (d,), generator=g).to(torch.bfloat16) for _ in range(2)]
+    dev_ring = [t.to(cuda_device) for t in ring]
+    pos = torch.tensor(pos0, device=cuda_device)
+    cmc.window_append(*dev_ring, pos, *(t.to(cuda_device) for t in new))
+    for b, p in enumerate(pos0):
+        for which in range(2):
+            if p >= 0:
+                ring[which][b, :, :, p % W] = new[which][b]
+            assert torch.equal(dev_ring[which][b].cpu(), ring[which][b]), (b, which)
+    assert pos.cpu().tolist() == [p + 1 if p >= 0 else p for p in pos0]
