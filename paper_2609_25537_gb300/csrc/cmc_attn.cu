@@ -8,7 +8,7 @@
 // per unit (at most one per tile, at most 8): m = 1 (the Llama- and
 // Mistral-shaped steps) gives one CTA per unit, nothing split; m >= 2 (long
 // units, few of them) gives thread-block clusters of m CTAs per unit, each
-// CTA taking a contiguous share of the unit's tiles: at the end every CTA
+// CTA taking every m-th of the unit's tiles: at the end every CTA
 // leaves its fp32 (max, sum, output) record in its own shared memory, and
 // after a cluster barrier each CTA merges a slice of the output columns from
 // all m records (distributed shared memory, log-sum-exp rescale).  More units
@@ -28,8 +28,8 @@
 // at position c ^ (row & 7) within its 128-byte line, so the consumers'
 // ldmatrix reads are conflict-free.  Rows that hold no key are masked, and
 // their V rows zeroed, so stale or unwritten memory never reaches the output.
-// The unit's query rows travel with each tile (1-D bulk copy) and a small
-// header written by the producer.  A stage is "full" when its TMA transaction
+// The unit's query rows travel with its first tile in a CTA (1-D bulk copy),
+// a small header written by the producer with each.  A stage is "full" when its TMA transaction
 // bytes (expect_tx / complete_tx) and its cp.async copies
 // (cp.async.mbarrier.arrive) have landed; four consumer warps, each owning 16
 // keys of a tile, compute
@@ -47,10 +47,22 @@
 //
 // K/V rows are read once per launch, so their loads carry an L2 evict-first
 // policy.  Before its grid dependency wait (programmatic dependent launch)
-// each CTA prefetches its first four box tiles into L2: CTAs that become
+// each CTA prefetches its first few box tiles into L2: CTAs that become
 // resident in free slots or in the slots of the previous launch's exiting
 // CTAs thus pull their first tiles from HBM while that launch drains, and the
 // evict-first stream of the running launch does not push them out again.
+//
+// What lies between that wait and the first tile's products is on every
+// launch's critical path, and was most of a small launch (clock64 stamps at
+// d = 128, three stages: 0.8 us of index arithmetic with 64-bit divisions, 1.0
+// us for one lane to issue twelve boxes, 0.45 us from pos to the first header,
+// with its 64-bit remainder; full at 2.5 us).  So a CTA's place in the work is
+// worked out before the wait, in 32 bits; one lane of each consumer warp
+// issues a quarter of the first stages' boxes; and pos is under way before
+// anything else.  With the merge's peer loads all in flight (see there), 16
+// steps of one layer went from 107 to 77 us at one sequence of 64 + 512 keys,
+// from 174 to 150 us at 16 sequences, and 32 steps of the Llama-3-8B shape from
+// 464 to 445 us (one stream, graph).
 //
 // The fused decode step also appends the new token: the producer copies the
 // new token's K/V rows next to the tile that holds its ring slot, a consumer
@@ -77,9 +89,9 @@ constexpr int kWarps = 4;      // consumer warps; each owns 16 keys of a tile
 constexpr int kThreads = 32 * kWarps;
 constexpr size_t kWsHeader = 256;
 constexpr int kHalfBytes = kTileKeys * 128;  // one 64-row x 128-byte swizzled box
+constexpr int kMetaSlots = 4;                // producer idx prefetch distance (tiles)
 // Largest cluster of CTAs that share one unit (the portable cluster size).
 constexpr int kMaxClusterCtas = 8;
-constexpr int kMetaSlots = 4;                // producer metadata prefetch distance (tiles)
 
 // fp32 partial record of one CTA's share of a unit: max[G], sum[G], then, from
 // a 16-byte aligned offset, the unnormalised output [G][d].
@@ -110,10 +122,11 @@ struct AttnParams {
   int tpu;                // tiles per unit: t1_tiles Tier-1 tiles, then the ring tiles
   int t1_tiles;           // ceil(k / 64)
   int rot;                // in-unit processing order: tile (j + rot) % tpu at position j
-  long long base;         // tiles per CTA (CTAs below `rem` take one more)
-  long long rem;
+  int LH;                 // units per sequence: L * Hkv
+  int base;               // granules per CTA (CTAs below `rem` take one more); cluster plan:
+  int rem;                // tiles of the unit per CTA of the cluster, likewise
   int cm;                 // > 0: clusters of cm CTAs share each unit (CTA j of the cluster
-                          // takes positions [j tpu / cm, (j+1) tpu / cm)); 0: flat split
+                          // takes positions j, j + cm, ...); 0: flat split
   int gran;               // flat split: tiles per granule (1, or tpu: whole units per CTA)
   float scale_log2;       // softmax scale * log2(e)
   long long rope_offset;  // rotary embedding (GQA-layer step): position of ring token 0
@@ -287,6 +300,9 @@ __device__ __forceinline__ void tma_prefetch_l2(const CUtensorMap* map, int col,
                "r"(col), "r"(row)
                : "memory");
 }
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* m) {
+  asm volatile("prefetch.tensormap [%0];\n" ::"l"(m) : "memory");
+}
 __device__ __forceinline__ void bulk_prefetch_l2(const void* src, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(src), "r"(bytes) : "memory");
 }
@@ -305,6 +321,11 @@ __device__ __forceinline__ void cluster_sync_all() {
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t cluster_id() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%clusterid.x;\n" : "=r"(r));
   return r;
 }
 __device__ __forceinline__ uint32_t peer_smem(uint32_t local_addr, uint32_t rank) {
@@ -355,11 +376,19 @@ enum { H_NROWS = 0, H_NEWSLOT = 1, H_NEWROW = 2, H_MASKED = 3, H_BADLO = 4, H_BA
 // 32 lanes hit distinct banks.
 __host__ __device__ constexpr int merge_row_floats(int D) { return D + 4; }
 
+// What the producer needs to issue one tile of a gathered Tier-1 -- the idx
+// entries of its 64 rows -- staged in shared memory by asynchronous 4-byte
+// copies kMetaSlots tiles ahead of their use, so the producer does not wait on
+// a global load for every tile.
+struct MetaSlot {
+  int32_t idx[kTileKeys];
+};
+
 template <int D, int G, int NST, bool ROPE>
 constexpr size_t attn_smem_bytes() {
   return 1024 /* alignment slack */ +
          static_cast<size_t>(NST) * (Stage<D, G, ROPE>::kBytes + Stage<D, G, ROPE>::kAuxBytes) +
-         kMetaSlots * (kTileKeys * 4 + 16) +
+         kMetaSlots * sizeof(MetaSlot) + 16 /* pos of the first sequence */ +
          static_cast<size_t>(kWarps) * (2 * 8 + G * merge_row_floats(D)) * sizeof(float);
 }
 
@@ -383,48 +412,37 @@ __device__ __forceinline__ long long rec_slot(const AttnParams& p, long long c, 
   return t > ut0 ? t - ut0 : 0;
 }
 
-// Unit coordinates of the tile at a position of the flattened (unit, j)
-// order, advanced one tile at a time so that the main loop does no integer
-// division.  Within a unit, position j holds key tile lt = (j + rot) % tpu:
-// the ring tiles come first, so a CTA's first loads need no idx entries.
+// The tile at a position of the flattened (unit, j) order, advanced one tile
+// at a time so that the main loop does no integer division.  Within a unit,
+// position j holds key tile lt = (j + rot) % tpu: ring tiles come first, so a
+// CTA's first loads need no idx entries.  A CTA of a cluster takes every
+// cm-th position of its one unit.  Units are numbered ((b L) + l) Hkv + g, so
+// a unit's query and output rows start at row u G of [B, L, Hq, d].
 struct TileCursor {
-  int u, j, lt, b, l, g;  // unit, position and key tile within it, the unit's (b, l, g)
-  __device__ __forceinline__ void init(long long t, const AttnParams& p) {
-    const int LH = p.L * p.Hkv;
-    u = static_cast<int>(t / p.tpu);
-    j = static_cast<int>(t - static_cast<long long>(u) * p.tpu);
+  int u, j, lt, b;  // unit, position and key tile within it, the unit's sequence
+  int left;         // units of sequence b from u on
+  __device__ __forceinline__ void init(int unit, int pos, const AttnParams& p) {
+    u = unit;
+    j = pos;
     lt = j + p.rot;
     if (lt >= p.tpu) lt -= p.tpu;
-    b = u / LH;
-    const int lg = u - b * LH;
-    l = lg / p.Hkv;
-    g = lg - l * p.Hkv;
+    b = static_cast<int>(static_cast<unsigned>(u) / static_cast<unsigned>(p.LH));
+    left = (b + 1) * p.LH - u;
   }
   __device__ __forceinline__ void next(const AttnParams& p) {
-    if (++j == p.tpu) {
+    if (p.cm > 0) {
+      j += p.cm;
+    } else if (++j == p.tpu) {
       j = 0;
       ++u;
-      if (++g == p.Hkv) {
-        g = 0;
-        if (++l == p.L) {
-          l = 0;
-          ++b;
-        }
+      if (--left == 0) {
+        left = p.LH;
+        ++b;
       }
     }
     lt = j + p.rot;
     if (lt >= p.tpu) lt -= p.tpu;
   }
-};
-
-// What the producer needs to issue one tile -- the idx entries of its 64 rows
-// (gathered Tier-1 tiles only) and pos of its sequence -- staged in shared
-// memory by asynchronous 4- and 8-byte copies kMetaSlots tiles ahead of their
-// use, so the producer never waits on a global load.
-struct MetaSlot {
-  int32_t idx[kTileKeys];
-  long long pos;
-  long long pad;
 };
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32_t src_bytes) {
@@ -434,6 +452,10 @@ __device__ __forceinline__ void cp_async16_hint(uint32_t dst, const void* src, u
                                                 uint64_t policy) {
   asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2, %3;\n" ::"r"(dst), "l"(src),
                "r"(src_bytes), "l"(policy));
+}
+__device__ __forceinline__ void cp_async16_all(uint32_t dst, const void* src, uint64_t policy) {
+  asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src),
+               "l"(policy));
 }
 // Adds one pending arrival to `bar` now and completes it once every cp.async
 // this thread issued so far has landed.
@@ -469,13 +491,11 @@ __device__ __forceinline__ void prefetch_meta(const AttnParams& p, const TileCur
         cp_async_4(smem_addr(&slot->idx[lane + 32 * e]), i < p.k ? irow + i : irow, i < p.k ? 4u : 0u);
       }
     }
-    if (lane == 0) cp_async_8(smem_addr(&slot->pos), p.pos + c.b);
   }
   cp_async_commit();
 }
 
 struct TileMeta {
-  long long pos;
   int idx_lo, idx_hi;  // idx entries of rows lane and lane + 32 (gathered tiles)
 };
 
@@ -499,7 +519,11 @@ __device__ __forceinline__ SeqState seq_state(const AttnParams& p, long long pos
   if (!q.bad) {
     if (FUSED) {
       q.count = static_cast<int>(pos + 1 < p.W ? pos + 1 : p.W);
-      q.new_slot = static_cast<int>(pos % p.W);
+      // a 32-bit remainder where it will do (the 64-bit one is a long call on
+      // the way to every launch's first tile)
+      q.new_slot = (pos >> 32) == 0
+                       ? static_cast<int>(static_cast<unsigned>(pos) % static_cast<unsigned>(p.W))
+                       : static_cast<int>(pos % p.W);
     } else {
       q.count = static_cast<int>(pos < p.W ? pos : p.W);
     }
@@ -507,10 +531,12 @@ __device__ __forceinline__ SeqState seq_state(const AttnParams& p, long long pos
   return q;
 }
 
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;\n" ::"r"(smem_addr(bar)),
-               "r"(bytes)
-               : "memory");
+// pos[b] through L2 (another CTA of this launch advances it once every reader
+// has counted itself; the kernel before may have advanced it).
+__device__ __forceinline__ long long ld_pos(const AttnParams& p, int b) {
+  long long v;
+  asm volatile("ld.global.cg.s64 %0, [%1];\n" : "=l"(v) : "l"(p.pos + b) : "memory");
+  return v;
 }
 
 // Rotary embedding of a GQA-layer step: (cos, sin) of the angle
@@ -546,60 +572,33 @@ __device__ __forceinline__ void rope_pairs(const AttnParams& p, long long pos,
   }
 }
 
-// Producer lane 0, box tiles: what does not depend on pos -- the K/V boxes and
-// the unit's query rows -- issued as soon as the stage is free.  Two-
-// dimensional boxes of 64 consecutive rows of the ring, or of the Tier-1
-// tensor under identity selection; rows past the unit's keys are masked later,
-// rows past the tensor are zero-filled by the TMA unit.
-template <int D, int G>
-__device__ __forceinline__ void issue_box_loads(const AttnParams& p, const AttnMaps& maps,
-                                                uint8_t* stage, uint8_t* aux, const TileCursor& c,
-                                                uint64_t* full) {
-  using S = Stage<D, G>;
-  constexpr int H = S::kHalves;
-  const bool t1 = c.lt < p.t1_tiles;
-  const int row = t1 ? c.u * p.N + c.lt * kTileKeys : c.u * p.W + (c.lt - p.t1_tiles) * kTileKeys;
-  const CUtensorMap* mk = t1 ? &maps.t1k_box : &maps.rk_box;
-  const CUtensorMap* mv = t1 ? &maps.t1v_box : &maps.rv_box;
-  const uint32_t sK = smem_addr(stage + S::kK);
-  const uint32_t sV = smem_addr(stage + S::kV);
-  mbar_expect_tx(full, 2 * H * kHalfBytes + G * D * 2);
-  // K/V rows are read once per step: evict-first keeps them from displacing
-  // what is worth keeping in L2 (the prefetched first tiles of the next launch)
-  const uint64_t pol = policy_evict_first();
-#pragma unroll
-  for (int h = 0; h < H; ++h) {
-    tma_box_hint(sK + h * kHalfBytes, mk, h * 64, row, full, pol);
-    tma_box_hint(sV + h * kHalfBytes, mv, h * 64, row, full, pol);
-  }
-  const uint16_t* qsrc =
-      p.q + ((static_cast<long long>(c.b) * p.L + c.l) * p.Hq + static_cast<long long>(c.g) * G) * D;
-  bulk_copy(smem_addr(aux + S::kQ), qsrc, G * D * 2, full);
+// A box tile's K and V rows are 2 d / 64 boxes of 64 consecutive rows of the
+// ring, or of the Tier-1 tensor under identity selection; rows past the unit's
+// keys are masked later, rows past the tensor are zero-filled by the TMA unit.
+// Box w: K for w < d / 64, then V; its map, its first tensor column and row,
+// and its offset in the stage.
+template <int D>
+struct Boxes {
+  static constexpr int H = D / 64;
+  static constexpr int kCount = 2 * H;
+  static constexpr int kTx = kCount * kHalfBytes;  // bytes of a tile's boxes
+};
+__device__ __forceinline__ int box_row(const AttnParams& p, const TileCursor& c) {
+  return c.lt < p.t1_tiles ? c.u * p.N + c.lt * kTileKeys
+                           : c.u * p.W + (c.lt - p.t1_tiles) * kTileKeys;
 }
-
-// Producer lane 0, before the grid dependency wait: the boxes of a box tile
-// (and, for the first tile of a unit, the unit's query rows) prefetched into
-// L2.  A CTA that becomes resident while the previous kernel on the stream is
-// still running (a free slot, or one that kernel's exiting CTAs freed) thus
-// pulls its first tile from HBM during that kernel's tail; its loads after
-// the wait then hit L2.
-template <int D, int G>
-__device__ __forceinline__ void prefetch_box_tile(const AttnParams& p, const AttnMaps& maps,
-                                                  const TileCursor& c, bool with_q) {
-  constexpr int H = D / 64;
-  const bool t1 = c.lt < p.t1_tiles;
-  const int row = t1 ? c.u * p.N + c.lt * kTileKeys : c.u * p.W + (c.lt - p.t1_tiles) * kTileKeys;
-  const CUtensorMap* mk = t1 ? &maps.t1k_box : &maps.rk_box;
-  const CUtensorMap* mv = t1 ? &maps.t1v_box : &maps.rv_box;
-#pragma unroll
-  for (int h = 0; h < H; ++h) {
-    tma_prefetch_l2(mk, h * 64, row);
-    tma_prefetch_l2(mv, h * 64, row);
-  }
-  if (with_q)
-    bulk_prefetch_l2(p.q + ((static_cast<long long>(c.b) * p.L + c.l) * p.Hq +
-                            static_cast<long long>(c.g) * G) * D,
-                     G * D * 2);
+template <int D>
+__device__ __forceinline__ const CUtensorMap* box_map(const AttnParams& p, const AttnMaps& maps,
+                                                      const TileCursor& c, int w) {
+  const bool v = w >= Boxes<D>::H;
+  return c.lt < p.t1_tiles ? (v ? &maps.t1v_box : &maps.t1k_box) : (v ? &maps.rv_box : &maps.rk_box);
+}
+template <int D>
+__device__ __forceinline__ void issue_box(const AttnParams& p, const AttnMaps& maps, uint32_t stage,
+                                          const TileCursor& c, int w, uint64_t* full,
+                                          uint64_t policy) {
+  tma_box_hint(stage + w * kHalfBytes, box_map<D>(p, maps, c, w), (w % Boxes<D>::H) * 64,
+               box_row(p, c), full, policy);
 }
 
 // Producer warp, once pos (and, for a gathered tile, its idx entries) is
@@ -607,9 +606,12 @@ __device__ __forceinline__ void prefetch_box_tile(const AttnParams& p, const Att
 // the new token's row), the new token's K/V rows in the fused step, the loads
 // of a gathered tile, and the arrive that, once every byte has landed,
 // releases the stage to the consumers.
+// The boxes of a box tile are on their way already, and may have landed: a
+// transaction count that runs below zero for a while is within its range, and
+// the phase cannot complete before this arrive.
 template <int D, int G, bool FUSED, bool ROPE>
 __device__ __forceinline__ void finish_tile(const AttnParams& p, uint8_t* stage, uint8_t* aux,
-                                            const TileCursor& c, const TileMeta& meta,
+                                            const TileCursor& c, bool with_q, const TileMeta& meta,
                                             const SeqState& sq, const float2 (&rope)[2], int lane,
                                             uint64_t* full) {
   using S = Stage<D, G, ROPE>;
@@ -632,9 +634,9 @@ __device__ __forceinline__ void finish_tile(const AttnParams& p, uint8_t* stage,
   const bool gath = t1 && p.idx != nullptr;
   if (gath) {
     // Tier-1 rows gathered by idx: 16-byte cp.async copies by the producer
-    // lanes (d/8 lanes sweep a row) to the swizzled positions; rows past k and
-    // rows with an out-of-range index are zero-filled.  Each lane's copies
-    // reach the full barrier through cp.async.mbarrier.arrive.
+    // lanes (d/8 lanes sweep a row) to the swizzled positions; rows with an
+    // out-of-range index are zero-filled.  Each lane's copies reach the full
+    // barrier through cp.async.mbarrier.arrive.
     constexpr int LPR = D / 8;     // lanes per row
     constexpr int RPP = 32 / LPR;  // rows per pass
     const uint32_t sK = smem_addr(stage + S::kK);
@@ -642,20 +644,65 @@ __device__ __forceinline__ void finish_tile(const AttnParams& p, uint8_t* stage,
     const int chunk = lane % LPR;
     const int rsub = lane / LPR;
     const long long ubase = static_cast<long long>(c.u) * p.N * D + chunk * 8;
+    const uint16_t* gk = p.t1k + ubase;
+    const uint16_t* gv = p.t1v + ubase;
     const uint64_t pol = policy_evict_first();
-#pragma unroll 8
-    for (int jj = 0; jj < kTileKeys / RPP; ++jj) {
-      const int r = jj * RPP + rsub;
-      const int row = __shfl_sync(0xffffffffu, (jj * RPP < 32) ? meta.idx_lo : meta.idx_hi, r & 31);
-      const bool ok = r < n_rows && static_cast<unsigned>(row) < static_cast<unsigned>(p.N);
-      const long long e = ubase + static_cast<long long>(ok ? row : 0) * D;
-      const uint32_t off = swz(r, chunk);
-      cp_async16_hint(sK + off, p.t1k + e, ok ? 16u : 0u, pol);
-      cp_async16_hint(sV + off, p.t1v + e, ok ? 16u : 0u, pol);
-    }
-    mbar_arrive_cp_async(full);
     bad_lo = __ballot_sync(0xffffffffu, lane < n_rows && static_cast<unsigned>(meta.idx_lo) >= static_cast<unsigned>(p.N));
     bad_hi = __ballot_sync(0xffffffffu, lane + 32 < n_rows && static_cast<unsigned>(meta.idx_hi) >= static_cast<unsigned>(p.N));
+    if (!(bad_lo | bad_hi)) {
+      // Every index is in range.  One warp issues the 64 d/4 copies of a tile
+      // and is what bounds a launch with many gathered tiles, so the loop
+      // holds little else: row r = RPP jj + rsub has r & 7 = (RPP jj & 7) |
+      // rsub, so its swizzled chunk repeats every 8 / RPP passes and the
+      // destinations are that many registers plus constants.  Passes past
+      // the tile's rows are left out, and the rows the last ones have over
+      // (their entries are zero: row 0) are masked like all rows without a
+      // key.  16 sequences of 1,024 + 512 keys, gathered: 19.6 us a step, from
+      // 26.2 with the general loop below; 32 layers of 128 + 512 keys in four
+      // streams end to end 14.4 us, from 15.1.
+      constexpr int P = 8 / RPP;
+      uint32_t dst[P];
+#pragma unroll
+      for (int q = 0; q < P; ++q) dst[q] = sK + swz(q * RPP + rsub, chunk);
+      if (n_rows == kTileKeys) {  // straight through: 4 % less for a launch of gathered tiles
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+          const int mine = half ? meta.idx_hi : meta.idx_lo;
+#pragma unroll
+          for (int jj = 0; jj < 32 / RPP; ++jj) {
+            const int row = __shfl_sync(0xffffffffu, mine, jj * RPP + rsub);
+            const uint32_t to = dst[jj % P] + (half * 32 + jj / P * 8) * 128;
+            const long long e = static_cast<long long>(row) * D;
+            cp_async16_all(to, gk + e, pol);
+            cp_async16_all(to + (S::kV - S::kK), gv + e, pol);
+          }
+        }
+      } else {
+        for (int r0 = 0; r0 < n_rows; r0 += 8 * RPP) {  // eight passes at a time
+          const int mine = r0 < 32 ? meta.idx_lo : meta.idx_hi;
+#pragma unroll
+          for (int jj = 0; jj < 8; ++jj) {
+            const int row = __shfl_sync(0xffffffffu, mine, (r0 & 31) + jj * RPP + rsub);
+            const uint32_t to = dst[jj % P] + (r0 + jj / P * 8) * 128;
+            const long long e = static_cast<long long>(row) * D;
+            cp_async16_all(to, gk + e, pol);
+            cp_async16_all(to + (S::kV - S::kK), gv + e, pol);
+          }
+        }
+      }
+    } else {
+#pragma unroll 1
+      for (int jj = 0; jj < kTileKeys / RPP; ++jj) {
+        const int r = jj * RPP + rsub;
+        const int row = __shfl_sync(0xffffffffu, (jj * RPP < 32) ? meta.idx_lo : meta.idx_hi, r & 31);
+        const bool ok = r < n_rows && static_cast<unsigned>(row) < static_cast<unsigned>(p.N);
+        const long long e = static_cast<long long>(ok ? row : 0) * D;
+        const uint32_t off = swz(r, chunk);
+        cp_async16_hint(sK + off, gk + e, ok ? 16u : 0u, pol);
+        cp_async16_hint(sV + off, gv + e, ok ? 16u : 0u, pol);
+      }
+    }
+    mbar_arrive_cp_async(full);
     __syncwarp();
   }
   if (lane == 0) {
@@ -668,15 +715,11 @@ __device__ __forceinline__ void finish_tile(const AttnParams& p, uint8_t* stage,
     hw[H_MASKED] = (n_rows < kTileKeys || (bad_lo | bad_hi)) ? 1 : 0;
     hw[H_BADLO] = static_cast<int>(bad_lo);
     hw[H_BADHI] = static_cast<int>(bad_hi);
-    uint32_t tx = p.stall_tx;   // 0 outside the failure-path test
-    if (gath) tx += G * D * 2;  // query rows (box tiles: issued with the boxes)
+    uint32_t tx = p.stall_tx;             // 0 outside the failure-path test
+    if (!gath) tx += Boxes<D>::kTx;       // the boxes
+    if (with_q) tx += G * D * 2;          // the unit's query rows (its first tile in this CTA)
     if (new_row >= 0) tx += 2 * D * 2;
     mbar_arrive_expect_tx(full, tx);  // releases the header
-    if (gath) {
-      const uint16_t* qsrc =
-          p.q + ((static_cast<long long>(c.b) * p.L + c.l) * p.Hq + static_cast<long long>(c.g) * G) * D;
-      bulk_copy(smem_addr(aux + S::kQ), qsrc, G * D * 2, full);
-    }
     if (new_row >= 0) {
       bulk_copy(smem_addr(aux + S::kNew), p.k_new + static_cast<long long>(c.u) * D, D * 2, full);
       bulk_copy(smem_addr(aux + S::kNew + D * 2), p.v_new + static_cast<long long>(c.u) * D, D * 2, full);
@@ -687,9 +730,9 @@ __device__ __forceinline__ void finish_tile(const AttnParams& p, uint8_t* stage,
 // Fused step: a CTA has read pos[b] for its run of `tiles` tiles of sequence
 // b.  The run that brings the sequence's count to all of its tiles is the last
 // reader of pos[b]; it advances pos[b] and clears the count for the next call.
-__device__ __forceinline__ void seq_run_done(const AttnParams& p, int b, long long tiles,
+__device__ __forceinline__ void seq_run_done(const AttnParams& p, int b, int tiles,
                                              const SeqState& sq) {
-  const unsigned long long total = static_cast<unsigned long long>(p.L) * p.Hkv * p.tpu;
+  const unsigned long long total = static_cast<unsigned long long>(p.LH) * p.tpu;
   const unsigned long long old = atomicAdd(p.tickets + b, static_cast<unsigned long long>(tiles));
   if (old + static_cast<unsigned long long>(tiles) == total) {
     if (!sq.bad) p.pos[b] = sq.pos + 1;
@@ -702,7 +745,7 @@ __device__ __forceinline__ void seq_run_done(const AttnParams& p, int b, long lo
 // full[s] (its bytes have landed and its header is written) and handed back
 // by empty[s] (every consumer warp is done with it).
 template <int D, int G, bool FUSED, int NST, bool ROPE>
-__global__ void __launch_bounds__(kThreads + 32)
+__global__ void __launch_bounds__(kThreads + 32, D == 64 ? 4 : 2)
 two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) {
   using S = Stage<D, G, ROPE>;
   constexpr int KS = D / 16;  // k-steps of the Q K^T product
@@ -711,7 +754,7 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* aux0 = smem + NST * S::kBytes;                              // NST aux areas
   uint8_t* meta0 = aux0 + NST * S::kAuxBytes;                          // kMetaSlots slots
-  float* merge_m = reinterpret_cast<float*>(meta0 + kMetaSlots * sizeof(MetaSlot));  // [kWarps][8]
+  float* merge_m = reinterpret_cast<float*>(meta0 + kMetaSlots * sizeof(MetaSlot) + 16);  // [kWarps][8]
   float* merge_l = merge_m + kWarps * 8;                               // [kWarps][8]
   float* merge_o = merge_l + kWarps * 8;                               // [kWarps][G][D]
   __shared__ __align__(8) uint64_t full_bar[NST];
@@ -721,18 +764,29 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
   const int lane = tid & 31;
   const int warp = tid >> 5;
 
-  const long long cta = blockIdx.x;
-  long long t_begin, t_end;
-  if (p.cm > 0) {  // clusters of cm CTAs per unit
-    const long long u = cta / p.cm;
-    const int j = static_cast<int>(cta - u * p.cm);
-    t_begin = u * p.tpu + (static_cast<long long>(j) * p.tpu) / p.cm;
-    t_end = u * p.tpu + (static_cast<long long>(j + 1) * p.tpu) / p.cm;
-  } else {
-    t_begin = cta_first_tile(cta, p.base, p.rem) * p.gran;
-    t_end = t_begin + (p.base + (cta < p.rem ? 1 : 0)) * p.gran;
+  // This CTA's first tile and its tiles, in order.
+  int u_begin, j_begin = 0, n_tiles;
+  {
+    const int cta = static_cast<int>(blockIdx.x);
+    if (p.cm > 0) {  // clusters of cm CTAs per unit
+      u_begin = static_cast<int>(cluster_id());
+      j_begin = static_cast<int>(cluster_ctarank());
+      n_tiles = p.base + (j_begin < p.rem ? 1 : 0);
+    } else {
+      const int first = cta * p.base + min(cta, p.rem);
+      const int n = p.base + (cta < p.rem ? 1 : 0);
+      if (p.gran > 1) {  // whole units
+        u_begin = first;
+        n_tiles = n * p.gran;
+      } else {
+        u_begin = static_cast<int>(static_cast<unsigned>(first) / static_cast<unsigned>(p.tpu));
+        j_begin = first - u_begin * p.tpu;
+        n_tiles = n;
+      }
+    }
   }
-  const int n_tiles = static_cast<int>(t_end - t_begin);
+  TileCursor c0;
+  c0.init(u_begin, j_begin, p);
 
   if (tid == 0) {
     for (int s = 0; s < NST; ++s) {
@@ -743,20 +797,36 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   __syncthreads();
-  if (warp == kWarps && lane == 0 && p.l2_prefetch > 0) {
-    asm volatile("prefetch.tensormap [%0];\n" ::"l"(&maps.rk_box) : "memory");
-    asm volatile("prefetch.tensormap [%0];\n" ::"l"(&maps.rv_box) : "memory");
-    if (p.idx == nullptr && p.k > 0) {
-      asm volatile("prefetch.tensormap [%0];\n" ::"l"(&maps.t1k_box) : "memory");
-      asm volatile("prefetch.tensormap [%0];\n" ::"l"(&maps.t1v_box) : "memory");
-    }
-    TileCursor cp;
-    cp.init(t_begin, p);
+  // The boxes of the CTA's first tiles are prefetched into L2 before the grid
+  // dependency wait, and loaded right after it, by one lane of each consumer
+  // warp, a box number a warp: a lane takes about 0.08 us for a box (the
+  // producer's lane 0 took 1.0 us for three tiles), and the consumers have
+  // nothing else to do yet.
+  constexpr int NBOX = Boxes<D>::kCount;
+  const bool boxer = warp < NBOX && lane == 0;
+  if (boxer) {
+    const bool v = warp >= Boxes<D>::H;
+    prefetch_map(v ? &maps.rv_box : &maps.rk_box);
+    if (p.idx == nullptr && p.k > 0) prefetch_map(v ? &maps.t1v_box : &maps.t1k_box);
+    TileCursor cp = c0;
     const int npf = n_tiles < p.l2_prefetch ? n_tiles : p.l2_prefetch;
     for (int i = 0; i < npf; ++i) {
-      if (!gathered_tile(p, cp)) prefetch_box_tile<D, G>(p, maps, cp, i == 0 || cp.j == 0);
+      if (!gathered_tile(p, cp))
+        tma_prefetch_l2(box_map<D>(p, maps, cp, warp), (warp % Boxes<D>::H) * 64, box_row(p, cp));
       cp.next(p);
     }
+  }
+  // the producer: the unit's query rows, and the sequence of the CTA's last
+  // tile (how far pos is read ahead)
+  int last_b = c0.b;
+  if (warp == kWarps) {
+    if (lane == 0 && p.l2_prefetch > 0)
+      bulk_prefetch_l2(p.q + static_cast<long long>(c0.u) * (G * D), G * D * 2);
+    if (p.cm == 0 && n_tiles > p.tpu)
+      last_b = static_cast<int>(static_cast<unsigned>(c0.u + (c0.j + n_tiles - 1) / p.tpu) /
+                                static_cast<unsigned>(p.LH));
+    else if (p.cm == 0 && c0.j + n_tiles > p.tpu && c0.left == 1)
+      last_b = c0.b + 1;
   }
   // The producer lanes' rotary frequencies from their device table (written
   // long before this launch, never by the kernel before it).
@@ -773,38 +843,30 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
 
   if (warp == kWarps) {
     // ======================= producer warp =======================
-    if (lane == 0) {
-      asm volatile("prefetch.tensormap [%0];\n" ::"l"(&maps.rk_box) : "memory");
-      asm volatile("prefetch.tensormap [%0];\n" ::"l"(&maps.rv_box) : "memory");
-      if (p.idx == nullptr && p.k > 0) {
-        asm volatile("prefetch.tensormap [%0];\n" ::"l"(&maps.t1k_box) : "memory");
-        asm volatile("prefetch.tensormap [%0];\n" ::"l"(&maps.t1v_box) : "memory");
-      }
-    }
-    TileCursor cm, ci;  // tile whose metadata is prefetched, tile issued
-    cm.init(t_begin, p);
-    ci = cm;
     MetaSlot* slots = reinterpret_cast<MetaSlot*>(meta0);
-#pragma unroll
-    for (int m = 0; m < kMetaSlots; ++m) {
-      prefetch_meta(p, cm, m < n_tiles, lane, &slots[m]);
-      cm.next(p);
+    // pos of the first sequence, then the query rows of the first unit
+    long long* pos_s = reinterpret_cast<long long*>(slots + kMetaSlots);
+    if (lane == 0) {
+      cp_async_8(smem_addr(pos_s), p.pos + c0.b);
+      bulk_copy(smem_addr(aux0 + S::kQ), p.q + static_cast<long long>(c0.u) * (G * D), G * D * 2,
+                &full_bar[0]);
     }
-    {
-      // The box tiles of the first NST stages: their loads do not depend on
-      // pos, so they go out before any metadata has arrived.
-      TileCursor cl = ci;
-      for (int i = 0; i < NST && i < n_tiles; ++i) {
-        if (lane == 0 && !gathered_tile(p, cl))
-          issue_box_loads<D, G>(p, maps, smem + i * S::kBytes, aux0 + i * S::kAuxBytes, cl, &full_bar[i]);
-        cl.next(p);
+    cp_async_commit();
+    TileCursor cm = c0, ci = c0;  // tile whose idx entries are prefetched, tile issued
+    const bool meta_used = p.idx != nullptr;
+    if (meta_used) {
+#pragma unroll
+      for (int m = 0; m < kMetaSlots; ++m) {
+        prefetch_meta(p, cm, m < n_tiles, lane, &slots[m]);
+        cm.next(p);
       }
     }
+    int run_b = ci.b;         // sequence of the current run of tiles
+    long long pos_next = 0;   // pos of the sequence after it, ahead of its use
+    if (run_b < last_b) pos_next = ld_pos(p, run_b + 1);
     int issued = 0;
-    int run_b = -1;           // sequence of the current run of tiles
-    long long run_tiles = 0;  // tiles in that run so far
+    int run_tiles = 0;        // tiles in that run so far
     SeqState sq;
-    sq.pos = 0; sq.count = 0; sq.new_slot = -1; sq.bad = true;
     float2 rope[2] = {make_float2(1.f, 0.f), make_float2(1.f, 0.f)};
     unsigned long long turns[2] = {0ull, 0ull};  // this lane's rotary frequencies (ROPE)
     if (ROPE) {
@@ -816,8 +878,14 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
         if (lane + 32 < D / 2) turns[1] = p.rope_turns[lane + 32];
       }
     }
+    if (meta_used) cp_async_wait<kMetaSlots>();
+    else cp_async_wait<0>();
+    __syncwarp();  // pos has landed
+    sq = seq_state<FUSED>(p, *pos_s);
+    if (ROPE && !sq.bad) rope_pairs<D>(p, sq.pos, turns, lane, rope);
     for (int i = 0; i < n_tiles; ++i) {
       const int s = i % NST;
+      const bool with_q = i == 0 || (p.cm == 0 && ci.j == 0);  // a unit's first tile in this CTA
       if (i >= NST) {
         // Lane 0 waits for the consumers to release the stage; the warp barrier
         // orders the other lanes' copies into it after that, and the broadcast
@@ -827,37 +895,47 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
         __syncwarp();
         ok = __shfl_sync(0xffffffffu, ok, 0);
         if (!ok) break;
-        if (lane == 0 && !gathered_tile(p, ci))
-          issue_box_loads<D, G>(p, maps, smem + s * S::kBytes, aux0 + s * S::kAuxBytes, ci, &full_bar[s]);
+        if (lane == 0 && !gathered_tile(p, ci)) {
+          const uint64_t pol = policy_evict_first();
+#pragma unroll
+          for (int w = 0; w < NBOX; ++w)
+            issue_box<D>(p, maps, smem_addr(smem + s * S::kBytes), ci, w, &full_bar[s], pol);
+        }
       }
-      MetaSlot* ms = &slots[i % kMetaSlots];
-      cp_async_wait<kMetaSlots - 1>();  // this tile's metadata has landed
-      __syncwarp();
+      if (with_q && i > 0 && lane == 0)
+        bulk_copy(smem_addr(aux0 + s * S::kAuxBytes + S::kQ),
+                  p.q + static_cast<long long>(ci.u) * (G * D), G * D * 2, &full_bar[s]);
       TileMeta meta;
-      meta.pos = ms->pos;
       meta.idx_lo = meta.idx_hi = -1;
-      if (gathered_tile(p, ci)) {
-        meta.idx_lo = ms->idx[lane];
-        meta.idx_hi = ms->idx[lane + 32];
+      if (meta_used) {
+        cp_async_wait<kMetaSlots - 1>();  // this tile's idx entries have landed
+        __syncwarp();
+        if (gathered_tile(p, ci)) {
+          meta.idx_lo = slots[i % kMetaSlots].idx[lane];
+          meta.idx_hi = slots[i % kMetaSlots].idx[lane + 32];
+        }
       }
       if (ci.b != run_b) {  // a new sequence: pos-derived state, once per run
-        if (FUSED && run_b >= 0 && lane == 0) seq_run_done(p, run_b, run_tiles, sq);
+        if (FUSED && lane == 0) seq_run_done(p, run_b, run_tiles, sq);
         run_b = ci.b;
         run_tiles = 0;
-        sq = seq_state<FUSED>(p, meta.pos);
-        if (ROPE && !sq.bad) rope_pairs<D>(p, meta.pos, turns, lane, rope);
+        sq = seq_state<FUSED>(p, pos_next);
+        if (ROPE && !sq.bad) rope_pairs<D>(p, sq.pos, turns, lane, rope);
+        if (run_b < last_b) pos_next = ld_pos(p, run_b + 1);
       }
       ++run_tiles;
-      finish_tile<D, G, FUSED, ROPE>(p, smem + s * S::kBytes, aux0 + s * S::kAuxBytes, ci, meta, sq,
-                                     rope, lane, &full_bar[s]);
+      finish_tile<D, G, FUSED, ROPE>(p, smem + s * S::kBytes, aux0 + s * S::kAuxBytes, ci, with_q,
+                                     meta, sq, rope, lane, &full_bar[s]);
       ci.next(p);
       issued = i + 1;
-      __syncwarp();
-      prefetch_meta(p, cm, i + kMetaSlots < n_tiles, lane, ms);  // the slot just read
-      cm.next(p);
+      if (meta_used) {
+        __syncwarp();
+        prefetch_meta(p, cm, i + kMetaSlots < n_tiles, lane, &slots[i % kMetaSlots]);  // the slot just read
+        cm.next(p);
+      }
     }
-    if (FUSED && run_b >= 0 && issued == n_tiles && lane == 0) seq_run_done(p, run_b, run_tiles, sq);
-    cp_async_wait<0>();  // this lane's cp.async copies (metadata, gathered rows) have landed
+    if (FUSED && issued == n_tiles && lane == 0) seq_run_done(p, run_b, run_tiles, sq);
+    cp_async_wait<0>();  // this lane's cp.async copies (pos, idx entries, gathered rows) have landed
     // No CTA exits while bulk loads it issued may still be writing into its
     // shared memory.  Normally the consumers have waited for every stage but
     // the last few, and this wait for the last issued stage covers the rest
@@ -883,6 +961,19 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
   }
 
   // ======================= consumer warps =======================
+  // The boxes of the first NST stages: their loads do not depend on pos, so
+  // they go out before any of the producer's headers.
+  if (boxer) {
+    const uint64_t pol = policy_evict_first();
+    TileCursor cl = c0;
+#pragma unroll
+    for (int i = 0; i < NST; ++i) {
+      if (i < n_tiles && !gathered_tile(p, cl))
+        issue_box<D>(p, maps, smem_addr(smem + i * S::kBytes), cl, warp, &full_bar[i], pol);
+      cl.next(p);
+    }
+  }
+  __syncwarp();
   // Both products take the warp's 16 keys (S^T = K Q^T) or 16 rows of the
   // head dimension (O^T = V^T P^T) as the M rows of m16n8k16 and the query
   // heads of the group as the N = 8 columns, so no M row is padding.
@@ -894,9 +985,9 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
   const int gq = lane >> 2;
   const int tq = lane & 3;
   constexpr int MT = D / 16;  // m-tiles of O^T
-  TileCursor cc;
-  cc.init(t_begin, p);
+  TileCursor cc = c0;
   int cur_u = -1;
+  int first_j = 0;  // position of this CTA's first tile of the current unit
   uint32_t qa[KS][2];  // Q^T fragments (B operand): head gq, columns of k-step ks
   float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
   float o[MT][4];
@@ -963,6 +1054,7 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
 
     if (u != cur_u) {  // first tile of a unit in this CTA
       cur_u = u;
+      first_j = cc.j;
       const uint8_t* qs = aux + S::kQ;
       if (ROPE && gq < G && !dead) {
         // rotate the query: column c of the first half pairs with c + d/2,
@@ -1106,7 +1198,7 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
     if (lane == 0) mbar_arrive(&empty_bar[s]);  // this warp is done with stage s
 
     // ---- end of a unit within this CTA: merge warps, write out or a partial ----
-    const bool unit_end = (i + 1 == n_tiles) || (cc.j == p.tpu - 1);
+    const bool unit_end = (i + 1 == n_tiles) || (p.cm == 0 && cc.j == p.tpu - 1);
     if (unit_end) {
       // Merge the four warps' states of each head: every warp leaves its
       // running max, sum and unnormalised output (rows of DP floats, padded so
@@ -1138,10 +1230,8 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
 
       // The unit is whole in this CTA unless the CTA's tile range cuts it; a
       // cut unit's record goes to the slot of this CTA's first tile in it.
-      const long long ut0 = static_cast<long long>(u) * p.tpu;
-      const bool whole = ut0 >= t_begin && ut0 + p.tpu <= t_end;
-      const long long out_base =
-          ((static_cast<long long>(cc.b) * p.L + cc.l) * p.Hq + static_cast<long long>(cc.g) * G) * D;
+      const bool whole = p.cm == 0 && first_j == 0 && cc.j == p.tpu - 1;
+      const long long out_base = static_cast<long long>(u) * (G * D);
       constexpr int NGR = G * D / 4;                      // 4-column groups of the unit's output
       constexpr int XPT = (NGR + kThreads - 1) / kThreads;  // groups per thread
       const bool clus = !whole && p.cm > 0;
@@ -1177,7 +1267,7 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
           cls[xi] = Ls;
         } else {  // merged by two_tier_combine_kernel
           constexpr int PW = rec_floats(G, D);
-          float* rec = p.partials + (ut0 + (ut0 > t_begin ? 0 : t_begin - ut0)) * PW;
+          float* rec = p.partials + (static_cast<long long>(u) * p.tpu + first_j) * PW;
           if (c == 0) {
             rec[hh] = M;
             rec[G + hh] = Ls;
@@ -1217,21 +1307,47 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
         for (int x = x0 + tid; x < x1; x += kThreads) {
           const int hh = (4 * x) / D;
           const int c = (4 * x) % D;
-          float M = -INFINITY;
-          for (int r = 0; r < cm; ++r)
-            M = fmaxf(M, ld_peer_f32(peer_smem(rec_local + hh * 4, r)));
+          // The peers' values are requested kChunk ranks at a time before the
+          // first is used (in a loop over the ranks each load waited for the
+          // one before it: 1.5 to 2.0 us from the barrier to the end, now 1.2).
+          // All eight ranks at once where the registers are there.
+          constexpr int kChunk = D == 64 ? 2 : (G <= 4 ? kMaxClusterCtas : 4);
+          float pm[kMaxClusterCtas], pl[kMaxClusterCtas];
+          float4 po[kChunk];
+          auto load_out = [&](int r0) {
+#pragma unroll
+            for (int e = 0; e < kChunk; ++e)
+              if (r0 + e < cm)
+                po[e] = ld_peer_f4(peer_smem(rec_local, r0 + e) + (rec_out_offset(G) + hh * D + c) * 4);
+          };
+#pragma unroll
+          for (int r = 0; r < kMaxClusterCtas; ++r) {
+            pm[r] = -INFINITY;
+            if (r < cm) {
+              const uint32_t base = peer_smem(rec_local, r);
+              pm[r] = ld_peer_f32(base + hh * 4);
+              pl[r] = ld_peer_f32(base + (G + hh) * 4);
+            }
+          }
+          load_out(0);
+          float M = pm[0];
+#pragma unroll
+          for (int r = 1; r < kMaxClusterCtas; ++r) M = fmaxf(M, pm[r]);
           float Ls = 0.f;
           float4 O = make_float4(0.f, 0.f, 0.f, 0.f);
           if (M != -INFINITY) {
-            for (int r = 0; r < cm; ++r) {
-              const uint32_t base = peer_smem(rec_local, r);
-              const float f = ex2(ld_peer_f32(base + hh * 4) - M);
-              const float4 o4 = ld_peer_f4(base + (rec_out_offset(G) + hh * D + c) * 4);
-              Ls = fmaf(f, ld_peer_f32(base + (G + hh) * 4), Ls);
-              O.x = fmaf(f, o4.x, O.x);
-              O.y = fmaf(f, o4.y, O.y);
-              O.z = fmaf(f, o4.z, O.z);
-              O.w = fmaf(f, o4.w, O.w);
+#pragma unroll
+            for (int r = 0; r < kMaxClusterCtas; ++r) {
+              if (r > 0 && r % kChunk == 0) load_out(r);
+              if (r < cm) {
+                const float4 o4 = po[r % kChunk];
+                const float f = ex2(pm[r] - M);
+                Ls = fmaf(f, pl[r], Ls);
+                O.x = fmaf(f, o4.x, O.x);
+                O.y = fmaf(f, o4.y, O.y);
+                O.z = fmaf(f, o4.z, O.z);
+                O.w = fmaf(f, o4.w, O.w);
+              }
             }
           }
           const float inv = Ls > 0.f ? __frcp_rn(Ls) : 0.f;
@@ -1257,11 +1373,6 @@ two_tier_combine_kernel(const AttnParams p) {
   asm volatile("griddepcontrol.wait;\n" ::: "memory");  // the attention kernel's records
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   const int u = blockIdx.x;
-  const int LH = p.L * p.Hkv;
-  const int b = u / LH;
-  const int lg = u - b * LH;
-  const int l = lg / p.Hkv;
-  const int g = lg - l * p.Hkv;
   const long long ut0 = static_cast<long long>(u) * p.tpu;
   const long long c0 = cta_of_tile(ut0, p.base, p.rem);
   const long long c1 = cta_of_tile(ut0 + p.tpu - 1, p.base, p.rem);
@@ -1271,8 +1382,7 @@ two_tier_combine_kernel(const AttnParams p) {
   const int nrec = static_cast<int>(c1 - c0 + 1);
   constexpr int PW = rec_floats(G, D);
   const float* recs = p.partials + ut0 * PW;
-  const long long out_base =
-      ((static_cast<long long>(b) * p.L + l) * p.Hq + static_cast<long long>(g) * G) * D;
+  const long long out_base = static_cast<long long>(u) * (G * D);
   for (int x = threadIdx.x; x < G * D / 2; x += blockDim.x) {
     const int hh = (2 * x) / D;
     const int c = (2 * x) % D;
@@ -1557,6 +1667,15 @@ static int plan_attn(long long total_tiles, int tpu, AttnPlan* pl) {
     pl->rem = ru;
   }
   // Flat split: is any unit cut between CTAs (a CTA boundary inside a unit)?
+  if (units <= slots && pl->cm == 0) {  // one CTA per unit: whole units, one each
+    pl->gran = tpu;
+    pl->base = 1;
+    pl->rem = 0;
+  }
+  if (pl->cm > 0) {
+    pl->base = tpu / pl->cm;
+    pl->rem = tpu % pl->cm;
+  }
   pl->split = false;
   for (long long c = 1; pl->cm == 0 && pl->gran == 1 && c < ctas && !pl->split; ++c) {
     const long long t = c * pl->base + (c < pl->rem ? c : pl->rem);
@@ -1599,9 +1718,17 @@ static int launch_attn(const AttnMaps& maps, const AttnParams& p0, long long tot
   int st = plan_attn<D, G, FUSED, ROPE>(total_tiles, p0.tpu, &pl);
   if (st != CMC_OK) return st;
   AttnParams p = p0;
-  p.base = pl.base;
-  p.rem = pl.rem;
+  p.base = static_cast<int>(pl.base);
+  p.rem = static_cast<int>(pl.rem);
   p.cm = pl.cm;
+  if (p.idx) {
+    // Gathered Tier-1: each CTA begins with a pipeline's depth of ring tiles,
+    // which need no idx entries, then the gathered ones, whose rows come in
+    // more slowly, so that it does not end with them (32 layers of 128 + 512
+    // keys: 250 us a round of 16 steps, 259 with the gathered tiles last).
+    const int ring = p.tpu - p.t1_tiles, lead = kStages * (pl.cm > 0 ? pl.cm : 1);
+    p.rot = p.tpu - (ring < lead ? ring : lead);
+  }
   p.gran = pl.gran;
   st = launch_attn_kernel<D, G, FUSED, ROPE>(maps, p, pl, s);
   if (st != CMC_OK || !pl.split) return st;
@@ -1755,6 +1882,7 @@ static int run_attention(const void* q, const void* tier1_k, const void* tier1_v
   p.partials = reinterpret_cast<float*>(ws + w.partials_off);
   p.B = m.B; p.L = m.L; p.Hq = m.Hq; p.Hkv = m.Hkv; p.N = m.N; p.k = m.k; p.W = m.W;
   p.tpu = tpu;
+  p.LH = m.L * m.Hkv;
   p.t1_tiles = tier1_tiles(m);
   p.rot = p.t1_tiles % tpu;  // the first ring tile
   p.base = 0;

@@ -741,6 +741,30 @@ def test_l2_prefetch_depth_changes_no_result(cuda_device, tiles):
         np.testing.assert_array_equal(a, b)
 
 
+PARTIAL = [(1, 1), (15, 17), (16, 48), (30, 130), (48, 49), (63, 65), (65, 127), (100, 400)]
+
+
+@pytest.mark.parametrize("mode", MODES)
+@pytest.mark.parametrize("k,W", PARTIAL)
+@pytest.mark.parametrize("plan", ["cluster", "whole units"])
+def test_partial_tiles_and_partly_filled_rings(cuda_device, plan, k, W, mode):
+    """Sizes around the 16-row boxes of a partial tile and the 64-row tiles, with rings from empty
+    to wrapped, so that ring tiles without a key are left out in the middle of a launch: one
+    unit shared by a cluster, and several units and sequences in one CTA."""
+    fills = sorted({0, 1, 15, 16, 17, W // 3, W // 2, W - 1, W, 63, 64, 65} & set(range(W + 1)))
+    B, L = (len(fills), 1) if plan == "cluster" else (4 * len(fills), 16)
+    w = WORKLOADS["tiny"].with_(name="partial", B=B, L=L, N=128, k=k, W=W, T=3,
+                                W0=tuple(fills) * (B // len(fills)))
+    P = Problem(w, cuda_device, mode=mode)
+    for t in range(w.T):
+        out, ref = P.step(step_inputs(w, t))
+        assert_attn_close(to_f64(out), ref, f"step {t}")
+        # every sequence by itself: a short one weighs little in the batch's norm
+        for b in range(B):
+            assert_attn_close(to_f64(out[b]), ref[b], f"step {t}, sequence {b}")
+    P.check_state()
+
+
 @pytest.mark.parametrize("L,Hkv,d", [(1, 1, 64), (1, 128, 64), (1, 129, 64), (3, 43, 128),
                                      (16, 16, 128), (33, 16, 128), (80, 8, 128)])
 def test_window_append_one_cta_and_clusters(cuda_device, L, Hkv, d):
