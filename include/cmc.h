@@ -21,8 +21,8 @@
  *  - Every tensor argument is a DEVICE pointer to memory the caller owns.  The
  *    library allocates no memory and keeps no state between calls apart from
  *    the thread-local last CUDA error, a per-device SM-count cache, the
- *    per-device rotary frequency tables of cmc_decode_step_rope (written once
- *    per (theta, d)), the static score array of cmc_score_select_static and
+ *    rotary frequency tables of cmc_decode_step_rope (at most 16 on the host
+ *    and 16 per device, each written once per (theta, d)), the static score array of cmc_score_select_static and
  *    two process-wide settings of the attention launches
  *    (cmc_set_l2_prefetch_tiles, cmc_test_stall_attention_waits).
  *  - All work is enqueued on `stream` (a cudaStream_t passed as void*; NULL is

@@ -74,15 +74,25 @@ def _ranged(fn):
     return wrapped
 
 
-def _p(t: Optional[torch.Tensor]) -> ctypes.c_void_p:
-    return ctypes.c_void_p(0 if t is None else t.data_ptr())
+# The functions below are called once per decode step, so what they do on the
+# host counts: a step of a small decoder takes the GPU 5 us.  Pointers and
+# streams are passed to ctypes as plain integers (the argument types are
+# declared), the current stream is read without building a Stream object, and
+# a tensor that passes is looked at through as few attributes as will do.
+
+def _p(t: Optional[torch.Tensor]) -> int:
+    return 0 if t is None else t.data_ptr()
 
 
-def _stream(device: torch.device) -> ctypes.c_void_p:
-    return ctypes.c_void_p(torch.cuda.current_stream(device).cuda_stream)
+def _stream(device: torch.device) -> int:
+    index = device.index
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device() if index is None else index)
 
 
 def _need(t: torch.Tensor, name: str, dtype: torch.dtype, ndim: int, device=None) -> None:
+    if (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype is dtype and t.dim() == ndim
+            and t.is_contiguous() and (device is None or t.get_device() == device.index)):
+        return
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name} must be a torch.Tensor")
     if not t.is_cuda:
@@ -118,9 +128,8 @@ def denoise(emb: torch.Tensor, *, n_tokens: Optional[torch.Tensor] = None, g: in
             raise ValueError("n_tokens must be [B]")
     kept = torch.empty((B, n_max), dtype=torch.int32, device=dev)
     count = torch.empty(B, dtype=torch.int32, device=dev)
-    need = int(lib().cmc_denoise_workspace_size(B, n_max))
     if workspace is None:
-        workspace = _counter_workspace("denoise", need, dev)
+        workspace = _counter_workspace("denoise", int(lib().cmc_denoise_workspace_size(B, n_max)), dev)
     st = lib().cmc_denoise(_p(emb), _p(n_tokens), B, n_max, H, g, float(tau), keep_every,
                            _p(kept), _p(count), _p(workspace),
                            workspace.numel() * workspace.element_size(), _stream(dev))
@@ -172,7 +181,7 @@ _counter_ws_cache: Dict[Tuple, torch.Tensor] = {}
 def _counter_workspace(kind: str, nbytes: int, device: torch.device) -> torch.Tensor:
     """A zero-filled workspace, one per (kind, device, stream, size): its
     completion counters start at zero, and every call leaves them so."""
-    key = (kind, device.index, torch.cuda.current_stream(device).cuda_stream, nbytes)
+    key = (kind, device.index, _stream(device), nbytes)
     ws = _counter_ws_cache.get(key)
     if ws is None:
         ws = torch.zeros(nbytes, dtype=torch.uint8, device=device)
@@ -243,9 +252,9 @@ def question_select(question_tokens: torch.Tensor, cme_bank: torch.Tensor, k: in
     idx = torch.empty((B, k), dtype=torch.int32, device=dev)
     alpha = torch.empty(B, dtype=torch.int32, device=dev) if locate else None
     start = torch.empty(B, dtype=torch.int32, device=dev) if locate else None
-    need = int(lib().cmc_question_select_workspace_size(B, N))
     if workspace is None:
-        workspace = _counter_workspace("question", need, dev)
+        workspace = _counter_workspace(
+            "question", int(lib().cmc_question_select_workspace_size(B, N)), dev)
     st = lib().cmc_question_select(
         _p(question_tokens), _p(q_len), Lq, _p(cme_bank), B, N, D, k, _p(chunk_offset),
         _p(ctx_len), int(W or 0), _p(q_vec), _p(idx), _p(alpha), _p(start), _p(workspace),
@@ -260,6 +269,10 @@ def question_select(question_tokens: torch.Tensor, cme_bank: torch.Tensor, k: in
 
 def dims_of(q: torch.Tensor, tier1_k: torch.Tensor, idx: Optional[torch.Tensor],
             ring_k: torch.Tensor) -> CmcDims:
+    return CmcDims(*_sizes(q, tier1_k, idx, ring_k))
+
+
+def _sizes(q, tier1_k, idx, ring_k) -> Tuple:
     B, L, Hq, d = q.shape
     Bk, Lk, Hkv, N, dk = tier1_k.shape
     Br, Lr, Hr, W, dr = ring_k.shape
@@ -269,7 +282,7 @@ def dims_of(q: torch.Tensor, tier1_k: torch.Tensor, idx: Optional[torch.Tensor],
                          f"ring {tuple(ring_k.shape)}")
     if idx is not None and int(idx.shape[0]) != B:
         raise ValueError(f"idx shape {tuple(idx.shape)} does not match batch {B}")
-    return CmcDims(B, L, Hq, Hkv, d, N, k, W)
+    return B, L, Hq, Hkv, d, N, k, W
 
 
 def decode_attn_workspace_size(dims: CmcDims) -> int:
@@ -313,8 +326,9 @@ class DecodeWorkspace:
 _ws_cache: Dict[Tuple, DecodeWorkspace] = {}
 
 
-def _workspace_for(dims: CmcDims, device: torch.device) -> DecodeWorkspace:
-    key = (device.index, torch.cuda.current_stream(device).cuda_stream, dims.key())
+def _workspace_for(sizes: Tuple, dims: CmcDims, device: torch.device, stream: int
+                   ) -> DecodeWorkspace:
+    key = (device.index, stream, sizes)
     ws = _ws_cache.get(key)
     if ws is None:
         ws = DecodeWorkspace(dims, device)
@@ -334,15 +348,16 @@ def _attn_args(q, tier1_k, tier1_v, idx, ring_k, ring_v, pos, out):
         _need(idx, "idx", torch.int32, 2, dev)
     if tier1_v.shape != tier1_k.shape or ring_v.shape != ring_k.shape:
         raise ValueError("K and V tensors must have the same shapes")
-    dims = dims_of(q, tier1_k, idx, ring_k)
-    if int(pos.shape[0]) != dims.B:
-        raise ValueError(f"pos shape {tuple(pos.shape)} does not match batch {dims.B}")
+    sizes = _sizes(q, tier1_k, idx, ring_k)
+    if int(pos.shape[0]) != sizes[0]:
+        raise ValueError(f"pos shape {tuple(pos.shape)} does not match batch {sizes[0]}")
     if out is None:
         out = torch.empty_like(q)
-    _need(out, "out", torch.bfloat16, 4, dev)
-    if out.shape != q.shape:
-        raise ValueError("out must have the shape of q")
-    return dims, dev, out
+    else:
+        _need(out, "out", torch.bfloat16, 4, dev)
+        if out.shape != q.shape:
+            raise ValueError("out must have the shape of q")
+    return sizes, dev, out
 
 
 def _scale(scale: Optional[float]) -> float:
@@ -355,12 +370,14 @@ def two_tier_decode_attn(q, tier1_k, tier1_v, idx, ring_k, ring_v, pos, *,
                          workspace: Optional[DecodeWorkspace] = None) -> torch.Tensor:
     """Decode attention over [Tier-1 rows at idx | occupied ring slots]; see
     cmc_two_tier_decode_attn.  Returns bf16 [B, L, Hq, d]."""
-    dims, dev, out = _attn_args(q, tier1_k, tier1_v, idx, ring_k, ring_v, pos, out)
-    ws = workspace if workspace is not None else _workspace_for(dims, dev)
+    sizes, dev, out = _attn_args(q, tier1_k, tier1_v, idx, ring_k, ring_v, pos, out)
+    dims, stream = CmcDims(*sizes), _stream(dev)
+    ws = workspace if workspace is not None else _workspace_for(sizes, dims, dev, stream)
     st = lib().cmc_two_tier_decode_attn(
         _p(q), _p(tier1_k), _p(tier1_v), _p(idx), _p(ring_k), _p(ring_v), _p(pos),
-        ctypes.byref(dims), _scale(scale), _p(out), _p(ws.buf), ws.nbytes, _stream(dev))
-    check(st, "cmc_two_tier_decode_attn")
+        ctypes.byref(dims), _scale(scale), _p(out), _p(ws.buf), ws.nbytes, stream)
+    if st:
+        check(st, "cmc_two_tier_decode_attn")
     return out
 
 
@@ -375,25 +392,29 @@ def decode_step(q, tier1_k, tier1_v, idx, ring_k, ring_v, pos, k_new, v_new, *,
     With ``rope_theta`` the step is that of a real GQA layer (see
     cmc_decode_step_rope): q and k_new are given before rotary embedding and
     are rotated at position ``rope_offset + pos[b]`` inside the launch."""
-    dims, dev, out = _attn_args(q, tier1_k, tier1_v, idx, ring_k, ring_v, pos, out)
+    sizes, dev, out = _attn_args(q, tier1_k, tier1_v, idx, ring_k, ring_v, pos, out)
     _need(k_new, "k_new", torch.bfloat16, 4, dev)
     _need(v_new, "v_new", torch.bfloat16, 4, dev)
-    want = (dims.B, dims.L, dims.Hkv, dims.d)
-    if tuple(k_new.shape) != want or tuple(v_new.shape) != want:
+    B, L, _, Hkv, d = sizes[:5]
+    want = (B, L, Hkv, d)
+    if k_new.shape != want or v_new.shape != want:
         raise ValueError(f"k_new/v_new must be {want}")
-    ws = workspace if workspace is not None else _workspace_for(dims, dev)
+    dims, stream = CmcDims(*sizes), _stream(dev)
+    ws = workspace if workspace is not None else _workspace_for(sizes, dims, dev, stream)
     if rope_theta is None:
         st = lib().cmc_decode_step(
             _p(q), _p(tier1_k), _p(tier1_v), _p(idx), _p(ring_k), _p(ring_v), _p(pos),
             _p(k_new), _p(v_new), ctypes.byref(dims), _scale(scale), _p(out), _p(ws.buf),
-            ws.nbytes, _stream(dev))
-        check(st, "cmc_decode_step")
+            ws.nbytes, stream)
+        if st:
+            check(st, "cmc_decode_step")
     else:
         st = lib().cmc_decode_step_rope(
             _p(q), _p(tier1_k), _p(tier1_v), _p(idx), _p(ring_k), _p(ring_v), _p(pos),
             _p(k_new), _p(v_new), ctypes.byref(dims), _scale(scale), float(rope_theta),
-            int(rope_offset), _p(out), _p(ws.buf), ws.nbytes, _stream(dev))
-        check(st, "cmc_decode_step_rope")
+            int(rope_offset), _p(out), _p(ws.buf), ws.nbytes, stream)
+        if st:
+            check(st, "cmc_decode_step_rope")
     return out
 
 

@@ -1786,6 +1786,31 @@ static unsigned long long rope_turns_fixed(double theta, int i, int d) {
   return static_cast<unsigned long long>(t * 18446744073709551616.0L + 0.5L);  // t * 2^64
 }
 
+// The turns of all pairs of (theta, d), zero past d / 2.  The first kRopeSlots
+// pairs of values seen are kept: a call otherwise computes d / 2 long-double
+// powers, which where long double is a software format (Arm) is most of the
+// call.  Bounded, and guarded for calls from several threads.
+static void rope_turns_table(double theta, int d, unsigned long long (&out)[64]) {
+  static std::mutex mu;
+  static int n = 0;
+  static double thetas[kRopeSlots];
+  static int ds[kRopeSlots];
+  static unsigned long long tables[kRopeSlots][64];
+  std::lock_guard<std::mutex> lock(mu);
+  for (int i = 0; i < n; ++i)
+    if (thetas[i] == theta && ds[i] == d) {
+      memcpy(out, tables[i], sizeof(out));
+      return;
+    }
+  for (int i = 0; i < 64; ++i) out[i] = i < d / 2 ? rope_turns_fixed(theta, i, d) : 0ull;
+  if (n < kRopeSlots) {
+    memcpy(tables[n], out, sizeof(out));
+    thetas[n] = theta;
+    ds[n] = d;
+    ++n;
+  }
+}
+
 // The slot of g_rope_tables holding the table of (theta, d) on the current
 // device, writing it on first use; -1 (use the kernel parameters) when the
 // slots are full, the stream is being captured into a graph, or the copy
@@ -1894,8 +1919,8 @@ static int run_attention(const void* q, const void* tier1_k, const void* tier1_v
   p.rope_offset = rope ? rope_offset : 0;
   p.l2_prefetch = g_l2_prefetch_tiles.load(std::memory_order_relaxed);
   p.stall_tx = g_stall_tx.load(std::memory_order_relaxed);
-  for (int i = 0; i < 64; ++i)
-    p.rope_turns[i] = (rope && i < m.d / 2) ? rope_turns_fixed(rope_theta, i, m.d) : 0ull;
+  if (rope) rope_turns_table(rope_theta, m.d, p.rope_turns);
+  else memset(p.rope_turns, 0, sizeof(p.rope_turns));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   p.rope_slot = rope ? rope_slot(rope_theta, m.d, p.rope_turns, s) : -1;
   const int G = m.Hq / m.Hkv;
