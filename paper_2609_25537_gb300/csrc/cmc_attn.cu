@@ -8,15 +8,16 @@
 // per unit (at most one per tile, at most 8): m = 1 (the Llama- and
 // Mistral-shaped steps) gives one CTA per unit, nothing split; m >= 2 (long
 // units, few of them) gives thread-block clusters of m CTAs per unit, each
-// CTA taking every m-th of the unit's tiles: at the end every CTA
-// leaves its fp32 (max, sum, output) record in its own shared memory, and
-// after a cluster barrier each CTA merges a slice of the output columns from
-// all m records (distributed shared memory, log-sum-exp rescale).  More units
+// CTA taking every m-th of the unit's tiles: at the end every CTA stores its
+// fp32 (max, sum, output) into its peers' shared memory (asynchronous stores
+// counted by a barrier there), to each the slice of output columns that peer
+// merges (log-sum-exp rescale) and writes.  More units
 // than resident CTAs: one wave of CTAs, each taking a contiguous run of whole
 // units when that is balanced enough, else an equal share of the flattened
 // (unit, tile) list (stream-K) with partial records in global memory that a
 // small combine kernel following on the stream merges.  No CTA ever
-// waits on another outside its cluster's two barriers.
+// waits on another outside its cluster: one cluster barrier, arrived at on entry
+// and waited for before the first store, and one wait for the peers' stores.
 //
 // Inside a CTA one producer warp streams the tiles through a ring of shared-
 // memory stages.  Ring tiles, and Tier-1 tiles when the Tier-1 rows are the
@@ -127,6 +128,7 @@ struct AttnParams {
   int rem;                // tiles of the unit per CTA of the cluster, likewise
   int cm;                 // > 0: clusters of cm CTAs share each unit (CTA j of the cluster
                           // takes positions j, j + cm, ...); 0: flat split
+  int slice;              // cluster plan: 4-column output groups each CTA finishes
   int gran;               // flat split: tiles per granule (1, or tpu: whole units per CTA)
   float scale_log2;       // softmax scale * log2(e)
   long long rope_offset;  // rotary embedding (GQA-layer step): position of ring token 0
@@ -209,6 +211,7 @@ __device__ __forceinline__ uint32_t pack_bf16_rn(float lo, float hi) {
 // participation never depends on whether a wait succeeded (see the kernel),
 // so a CTA whose waits gave up still reaches its end.
 constexpr uint32_t kWaitNs = 1000000000u;  // 1 s: the kernel runs for microseconds
+constexpr uint32_t kPeerWaitNs = 3000000000u;  // for a cluster's other CTAs: see mbar_wait_peers
 constexpr uint32_t kDrainNs = 2000000u;    // after a timeout: wait for issued loads
 constexpr uint32_t kMaxWaitPolls = 1u << 28;
 
@@ -314,9 +317,15 @@ __device__ __forceinline__ void consumer_sync() {
 
 // --- thread-block cluster: barrier (every thread of every CTA of the
 // cluster arrives, then waits) and loads from a peer CTA's shared memory.
-__device__ __forceinline__ void cluster_sync_all() {
+__device__ __forceinline__ void cluster_arrive() {
   asm volatile("barrier.cluster.arrive.release;\n" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
   asm volatile("barrier.cluster.wait.acquire;\n" ::: "memory");
+}
+__device__ __forceinline__ void cluster_sync_all() {
+  cluster_arrive();
+  cluster_wait();
 }
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;
@@ -333,18 +342,42 @@ __device__ __forceinline__ uint32_t peer_smem(uint32_t local_addr, uint32_t rank
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(local_addr), "r"(rank));
   return r;
 }
-__device__ __forceinline__ float ld_peer_f32(uint32_t addr) {
-  float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];\n" : "=f"(v) : "r"(addr) : "memory");
-  return v;
+// Asynchronous stores into a peer CTA's shared memory, counted in bytes by a
+// barrier there.
+__device__ __forceinline__ void st_peer_f4(uint32_t addr, const float4& v, uint32_t bar) {
+  asm volatile(
+      "st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];\n" ::"r"(
+          addr),
+      "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(bar)
+      : "memory");
 }
-__device__ __forceinline__ float4 ld_peer_f4(uint32_t addr) {
-  float4 v;
-  asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];\n"
-               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-               : "r"(addr)
-               : "memory");
-  return v;
+__device__ __forceinline__ void st_peer_f2(uint32_t addr, float x, float y, uint32_t bar) {
+  asm volatile(
+      "st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];\n" ::"r"(
+          addr),
+      "f"(x), "f"(y), "r"(bar)
+      : "memory");
+}
+// Waits for the peers' stores counted by `bar` (phase 0).  Unlike the pipeline's
+// waits it does not end with the CTA's abort flag: a CTA must not leave while
+// its peers still store into its shared memory.  Peers that gave up have done
+// so within kWaitNs of the cluster's start and store all the same, so the
+// limit (kPeerWaitNs) lies well behind theirs.
+__device__ __forceinline__ bool mbar_wait_peers(uint64_t* bar) {
+  const uint32_t t0 = global_ns32();
+  for (uint32_t it = 0; it < kMaxWaitPolls; ++it) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n"
+        " selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(smem_addr(bar))
+        : "memory");
+    if (ok) return true;
+    if (global_ns32() - t0 > kPeerWaitNs) break;
+  }
+  *static_cast<volatile int*>(&attn_abort) = 1;
+  return false;
 }
 
 // ---------------------------------------------------------------------------
@@ -361,7 +394,7 @@ struct Stage {
   static constexpr int kQ = 0;                         // query rows [G][D] bf16
   static constexpr int kNew = G * D * 2;               // new token K row, V row (fused step)
   static constexpr int kHdr = kNew + 2 * D * 2;        // header words (H_*)
-  static constexpr int kRope = kHdr + 128;             // rotary table: d/2 (cos, sin) pairs
+  static constexpr int kRope = kHdr + 32;              // rotary table: d/2 (cos, sin) pairs
   static constexpr int kAuxBytes = kRope + (ROPE ? D * 4 : 0);
 };
 
@@ -369,7 +402,9 @@ struct Stage {
 // token's ring slot and tile row (fused step; -1 if not in this tile),
 // whether any of the 64 rows holds no key (its V row must be zeroed), and the
 // bit masks of rows 0-31 / 32-63 whose Tier-1 index is out of range.
-enum { H_NROWS = 0, H_NEWSLOT = 1, H_NEWROW = 2, H_MASKED = 3, H_BADLO = 4, H_BADHI = 5 };
+// Stage 0's also holds, in its last two words, pos of the CTA's first sequence
+// on its way to the producer.
+enum { H_NROWS = 0, H_NEWSLOT = 1, H_NEWROW = 2, H_MASKED = 3, H_BADLO = 4, H_BADHI = 5, H_POS = 6 };
 
 // Row length (floats) of the end-of-unit merge buffer: d + 4, so that the
 // rows of the four head pairs a warp stores to start 8 banks apart and its
@@ -384,11 +419,32 @@ struct MetaSlot {
   int32_t idx[kTileKeys];
 };
 
+// What a CTA of a cluster receives from its peers at the end of their unit: from
+// each rank (max, sum) of the G heads, and the unnormalised output of the
+// 4-column groups this CTA finishes, SL = ceil(G D / 4 / cm) of them.  The
+// groups fill the query areas of stages 1 and 2, which a cluster plan never
+// uses (its one unit's query rows come with the first tile, in stage 0: 2 x 2
+// G D bytes hold G D / 4 groups), and an own area for the cm - 1 more that cm
+// SL can be.
+template <int D, int G, bool ROPE>
+struct Recv {
+  static constexpr int kPerStage = G * D * 2 / 16;  // groups in one query area
+  static constexpr int kExtra = (kMaxClusterCtas - 2) * 16;  // (eight CTAs share G D / 4 evenly)
+  static constexpr int kBytes = kExtra + kMaxClusterCtas * G * 8;
+  // byte offset of group n from the aux areas' start; `extra` is the own area's
+  __device__ static __forceinline__ uint32_t group(int n, uint32_t extra) {
+    using S = Stage<D, G, ROPE>;
+    return n < kPerStage       ? S::kAuxBytes + S::kQ + n * 16
+           : n < 2 * kPerStage ? 2 * S::kAuxBytes + S::kQ + (n - kPerStage) * 16
+                               : extra + (n - 2 * kPerStage) * 16;
+  }
+};
+
 template <int D, int G, int NST, bool ROPE>
 constexpr size_t attn_smem_bytes() {
-  return 1024 /* alignment slack */ +
+  return 1008 /* alignment slack: the base is 16-byte aligned */ +
          static_cast<size_t>(NST) * (Stage<D, G, ROPE>::kBytes + Stage<D, G, ROPE>::kAuxBytes) +
-         kMetaSlots * sizeof(MetaSlot) + 16 /* pos of the first sequence */ +
+         kMetaSlots * sizeof(MetaSlot) + Recv<D, G, ROPE>::kBytes +
          static_cast<size_t>(kWarps) * (2 * 8 + G * merge_row_floats(D)) * sizeof(float);
 }
 
@@ -754,11 +810,14 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* aux0 = smem + NST * S::kBytes;                              // NST aux areas
   uint8_t* meta0 = aux0 + NST * S::kAuxBytes;                          // kMetaSlots slots
-  float* merge_m = reinterpret_cast<float*>(meta0 + kMetaSlots * sizeof(MetaSlot) + 16);  // [kWarps][8]
+  float* merge_m = reinterpret_cast<float*>(meta0 + kMetaSlots * sizeof(MetaSlot) +
+                                            Recv<D, G, ROPE>::kBytes);  // [kWarps][8]
   float* merge_l = merge_m + kWarps * 8;                               // [kWarps][8]
   float* merge_o = merge_l + kWarps * 8;                               // [kWarps][G][D]
   __shared__ __align__(8) uint64_t full_bar[NST];
   __shared__ __align__(8) uint64_t empty_bar[NST];
+  __shared__ __align__(8) uint64_t recv_bar;  // cluster plan: the peers' stores
+  static_assert(NST >= 3, "the receive areas lie in stages 1 and 2");
 
   const int tid = threadIdx.x;
   const int lane = tid & 31;
@@ -796,7 +855,16 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
     attn_abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
+  if (tid == 32 && p.cm > 0) {  // the groups this CTA finishes and the heads' (max, sum), from each rank
+    const int mine = min(max(G * D / 4 - j_begin * p.slice, 0), p.slice);
+    mbar_init(&recv_bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    mbar_arrive_expect_tx(&recv_bar, static_cast<uint32_t>(p.cm * (mine * 16 + G * 8)));
+  }
   __syncthreads();
+  // The cluster's only barrier: the receive barriers exist before a peer's
+  // first store.  Waited for just before those.
+  if (p.cm > 0) cluster_arrive();
   // The boxes of the CTA's first tiles are prefetched into L2 before the grid
   // dependency wait, and loaded right after it, by one lane of each consumer
   // warp, a box number a warp: a lane takes about 0.08 us for a box (the
@@ -845,7 +913,7 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
     // ======================= producer warp =======================
     MetaSlot* slots = reinterpret_cast<MetaSlot*>(meta0);
     // pos of the first sequence, then the query rows of the first unit
-    long long* pos_s = reinterpret_cast<long long*>(slots + kMetaSlots);
+    long long* pos_s = reinterpret_cast<long long*>(aux0 + S::kHdr + 4 * H_POS);
     if (lane == 0) {
       cp_async_8(smem_addr(pos_s), p.pos + c0.b);
       bulk_copy(smem_addr(aux0 + S::kQ), p.q + static_cast<long long>(c0.u) * (G * D), G * D * 2,
@@ -950,13 +1018,7 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
     }
     if (lane == 0 && attn_aborted()) atomicOr(p.status, CMC_DEVFLAG_TIMEOUT);
     __syncwarp();
-    // A cluster plan: the consumers of every CTA of the cluster pass two
-    // cluster barriers at the end of their (one) unit; this warp passes the
-    // same two, so every thread of the cluster arrives at each.
-    if (p.cm > 0) {
-      cluster_sync_all();
-      cluster_sync_all();
-    }
+    if (p.cm > 0) cluster_wait();  // every thread that arrived waits
     return;
   }
 
@@ -1236,7 +1298,7 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
       constexpr int XPT = (NGR + kThreads - 1) / kThreads;  // groups per thread
       const bool clus = !whole && p.cm > 0;
       float4 cacc[XPT];
-      float cls[XPT];
+      float cls[XPT], cmx[XPT];
 #pragma unroll
       for (int xi = 0; xi < XPT; ++xi) {
         const int x = tid + xi * kThreads;
@@ -1265,6 +1327,7 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
         } else if (clus) {  // merged across the cluster below
           cacc[xi] = acc;
           cls[xi] = Ls;
+          cmx[xi] = M;
         } else {  // merged by two_tier_combine_kernel
           constexpr int PW = rec_floats(G, D);
           float* rec = p.partials + (static_cast<long long>(u) * p.tpu + first_j) * PW;
@@ -1276,73 +1339,56 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
         }
       }
       if (clus) {
-        // Each CTA of the cluster holds one share of the unit.  Its (max, sum,
-        // output) record goes to its own shared memory (over the merge
-        // buffer, now read); after a cluster barrier every CTA merges a slice
-        // of the output columns from all the records (log-sum-exp rescale, in
-        // rank order) and writes them; a second barrier keeps each record
-        // alive until every peer has read it.
-        float* rec = merge_o;
-        consumer_sync();
+        // Each CTA of the cluster holds one share of the unit.  It stores its
+        // (max, sum, output) into its peers' receive areas, to each the output
+        // groups that peer finishes, and merges what its own peers sent
+        // (log-sum-exp rescale, in rank order) once its barrier has counted
+        // all of it.  That is one trip over the cluster where a barrier, loads
+        // and a barrier were three: 16 steps of the tiny shape 59.6 us instead
+        // of 67.6, of 16 sequences of 64 + 512 keys 146 instead of 151, of one
+        // sequence of 1,024 + 2,048 keys 123 instead of 128.
+        const int cm = p.cm;
+        const int rank = static_cast<int>(cluster_ctarank());
+        const int SL = p.slice;
+        const uint32_t extra = static_cast<uint32_t>(reinterpret_cast<uint8_t*>(merge_m) - aux0) -
+                               Recv<D, G, ROPE>::kBytes;
+        const uint32_t aux_a = smem_addr(aux0), bar_a = smem_addr(&recv_bar);
+        const uint32_t ml_a = aux_a + extra + Recv<D, G, ROPE>::kExtra;
+        cluster_wait();
 #pragma unroll
         for (int xi = 0; xi < XPT; ++xi) {
           const int x = tid + xi * kThreads;
           if (x >= NGR) break;
           const int hh = (4 * x) / D;
-          const int c = (4 * x) % D;
-          if (c == 0) {  // merge_m still holds the warps' maxima
-            float M = merge_m[hh];
-#pragma unroll
-            for (int w = 1; w < kWarps; ++w) M = fmaxf(M, merge_m[w * 8 + hh]);
-            rec[hh] = M;
-            rec[G + hh] = cls[xi];
+          const int to = x / SL;
+          st_peer_f4(peer_smem(aux_a + Recv<D, G, ROPE>::group(rank * SL + x - to * SL, extra), to),
+                     cacc[xi], peer_smem(bar_a, to));
+          if ((4 * x) % D == 0) {
+            for (int r = 0; r < cm; ++r)
+              st_peer_f2(peer_smem(ml_a + (rank * G + hh) * 8, r), cmx[xi], cls[xi], peer_smem(bar_a, r));
           }
-          *reinterpret_cast<float4*>(rec + rec_out_offset(G) + hh * D + c) = cacc[xi];
         }
-        cluster_sync_all();
-        const int cm = p.cm;
-        const int rank = static_cast<int>(cluster_ctarank());
-        const int x0 = (rank * NGR) / cm, x1 = ((rank + 1) * NGR) / cm;
-        const uint32_t rec_local = smem_addr(rec);
+        mbar_wait_peers(&recv_bar);
+        const int x0 = rank * SL, x1 = min(x0 + SL, NGR);
         for (int x = x0 + tid; x < x1; x += kThreads) {
           const int hh = (4 * x) / D;
           const int c = (4 * x) % D;
-          // The peers' values are requested kChunk ranks at a time before the
-          // first is used (in a loop over the ranks each load waited for the
-          // one before it: 1.5 to 2.0 us from the barrier to the end, now 1.2).
-          // All eight ranks at once where the registers are there.
-          constexpr int kChunk = D == 64 ? 2 : (G <= 4 ? kMaxClusterCtas : 4);
-          float pm[kMaxClusterCtas], pl[kMaxClusterCtas];
-          float4 po[kChunk];
-          auto load_out = [&](int r0) {
+          const float2* ml = reinterpret_cast<const float2*>(aux0 + extra + Recv<D, G, ROPE>::kExtra) + hh;
+          float M = -INFINITY;
 #pragma unroll
-            for (int e = 0; e < kChunk; ++e)
-              if (r0 + e < cm)
-                po[e] = ld_peer_f4(peer_smem(rec_local, r0 + e) + (rec_out_offset(G) + hh * D + c) * 4);
-          };
-#pragma unroll
-          for (int r = 0; r < kMaxClusterCtas; ++r) {
-            pm[r] = -INFINITY;
-            if (r < cm) {
-              const uint32_t base = peer_smem(rec_local, r);
-              pm[r] = ld_peer_f32(base + hh * 4);
-              pl[r] = ld_peer_f32(base + (G + hh) * 4);
-            }
-          }
-          load_out(0);
-          float M = pm[0];
-#pragma unroll
-          for (int r = 1; r < kMaxClusterCtas; ++r) M = fmaxf(M, pm[r]);
+          for (int r = 0; r < kMaxClusterCtas; ++r)
+            if (r < cm) M = fmaxf(M, ml[r * G].x);
           float Ls = 0.f;
           float4 O = make_float4(0.f, 0.f, 0.f, 0.f);
           if (M != -INFINITY) {
 #pragma unroll
             for (int r = 0; r < kMaxClusterCtas; ++r) {
-              if (r > 0 && r % kChunk == 0) load_out(r);
               if (r < cm) {
-                const float4 o4 = po[r % kChunk];
-                const float f = ex2(pm[r] - M);
-                Ls = fmaf(f, pl[r], Ls);
+                const float2 mr = ml[r * G];
+                const float4 o4 = *reinterpret_cast<const float4*>(
+                    aux0 + Recv<D, G, ROPE>::group(r * SL + x - x0, extra));
+                const float f = ex2(mr.x - M);
+                Ls = fmaf(f, mr.y, Ls);
                 O.x = fmaf(f, o4.x, O.x);
                 O.y = fmaf(f, o4.y, O.y);
                 O.z = fmaf(f, o4.z, O.z);
@@ -1354,7 +1400,6 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
           *reinterpret_cast<uint2*>(p.out + out_base + hh * D + c) =
               make_uint2(pack_bf16_rn(O.x * inv, O.y * inv), pack_bf16_rn(O.z * inv, O.w * inv));
         }
-        cluster_sync_all();
       }
       if (i + 1 < n_tiles) consumer_sync();  // merge buffers are reused by the next unit
     }
@@ -1721,6 +1766,7 @@ static int launch_attn(const AttnMaps& maps, const AttnParams& p0, long long tot
   p.base = static_cast<int>(pl.base);
   p.rem = static_cast<int>(pl.rem);
   p.cm = pl.cm;
+  p.slice = pl.cm > 0 ? (G * D / 4 + pl.cm - 1) / pl.cm : 0;
   if (p.idx) {
     // Gathered Tier-1: each CTA begins with a pipeline's depth of ring tiles,
     // which need no idx entries, then the gathered ones, whose rows come in
