@@ -58,3 +58,13 @@ def test_bridge_epilogue_below_the_cap_and_in_place(cuda_device):
 
 def test_bridge_epilogue_many_rows(cuda_device):
     _case(20000, 64, 0.5, 1.0, True, cuda_device, seed=9)
+
+
+@pytest.mark.parametrize("D,per_sm", [(4, 8), (2048, 8), (2052, 4), (4096, 4), (4100, 2), (8192, 2),
+                                      (8196, 1), (16384, 1)])
+@pytest.mark.parametrize("affine", [False, True])
+def test_bridge_epilogue_thread_counts(cuda_device, D, per_sm, affine):
+    """The row lengths where a CTA's threads change, over three more rows than the most CTAs
+    that are resident, so that some walk two (gamma and beta kept from the first)."""
+    sms = torch.cuda.get_device_properties(cuda_device).multi_processor_count
+    _case(per_sm * sms + 3, D, 0.8, 2.0, affine, cuda_device, in_place=True)
