@@ -880,16 +880,15 @@ score_select_fused_kernel(const __grid_constant__ FusedArgs a) {
   v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
   if ((lane & 1) == 0) part[warp][lane >> 1] = v[0];
   __syncthreads();
-  float qq = qq_part[0];
-#pragma unroll 4
-  for (int w = 1; w < kFusedWarps; ++w) qq += qq_part[w];
-  // warp r: row r's 32 warp sums, in the same butterfly; lane 0 writes the score
+  // warp r: row r's 32 warp sums, and the question's, in the same butterfly;
+  // lane 0 writes the score
   if (warp < R) {
-    float sd = part[lane][2 * warp], sm = part[lane][2 * warp + 1];
+    float sd = part[lane][2 * warp], sm = part[lane][2 * warp + 1], qq = qq_part[lane];
 #pragma unroll
     for (int off = 16; off >= 1; off >>= 1) {
       sd += __shfl_xor_sync(0xffffffffu, sd, off);
       sm += __shfl_xor_sync(0xffffffffu, sm, off);
+      qq += __shfl_xor_sync(0xffffffffu, qq, off);
     }
     if (lane == 0) {
       float sc = 0.f;
@@ -902,20 +901,23 @@ score_select_fused_kernel(const __grid_constant__ FusedArgs a) {
     }
   }
   __syncthreads();
-  if (tid == 0) {
-    if (a.la.sqnorm) {
-      // this CTA's largest squared norm (lowest index on ties, NaN lowest),
-      // raised into the sequence's argmax slot
-      unsigned long long top = 0ull;
-      for (int r = 0; r < R; ++r) {
-        const float v = rsq_s[r];
-        const unsigned long long key = isnan(v) ? 0ull : orderable(v);
-        const unsigned long long p =
-            (key << 32) | (0xFFFFFFFFu - static_cast<uint32_t>(r0 + r - b * a.N));
-        top = p > top ? p : top;
-      }
-      atomicMax(a.la.best + b, top);
+  unsigned long long top = 0ull;
+  if (a.la.sqnorm && warp == 0) {
+    // this CTA's largest squared norm (lowest index on ties, NaN lowest), a row
+    // a lane
+    if (lane < R) {
+      const float v = rsq_s[lane];
+      top = ((isnan(v) ? 0ull : static_cast<unsigned long long>(orderable(v))) << 32) |
+            (0xFFFFFFFFu - static_cast<uint32_t>(r0 + lane - b * a.N));
     }
+#pragma unroll
+    for (int off = kFusedRows / 2; off >= 1; off >>= 1) {
+      const unsigned long long u = __shfl_xor_sync(0xffffffffu, top, off);
+      top = u > top ? u : top;
+    }
+  }
+  if (tid == 0) {
+    if (a.la.sqnorm) atomicMax(a.la.best + b, top);  // raised into the sequence's argmax slot
     // acq_rel at GPU scope: releases the CTA's writes (they precede it through
     // the barrier, and this thread's raise in program order) and, for the
     // last CTA, acquires everyone else's
