@@ -183,8 +183,8 @@ CMC_API size_t cmc_score_select_workspace_size(int B, int N);
  * take one kernel launch: the CTA that writes the last score of a sequence (a
  * counter in the workspace tells it) selects that sequence's top k, starting
  * from the histogram the scoring CTAs built.  Larger
- * banks, or no workspace, take two launches (scoring, then selection).  Both
- * give the same selection.
+ * banks, or no workspace, take two launches (scoring, then selection; the
+ * histogram serves the second up to 32,768 CMEs).  All give the same selection.
  *
  * Scores are computed in fp32 with a fixed summation order, so equal rows get
  * bit-identical scores.  Equal scores go to the lower index; -0 equals +0.  A

@@ -10,13 +10,16 @@
 //
 // Larger banks, two launches:
 //  1. cosine_scores_kernel -- one CTA of 256 threads per CME row (grid-stride
-//     over rows): every thread streams its share of the row with 16-byte loads
+//     over rows), or cosine_scores_warp_kernel, one warp per row, for rows of
+//     up to 2,048 features: every thread streams its share of the row with 16-byte loads
 //     issued four at a time, accumulating m.q, m.m and q.q in fp32; the
 //     partial sums meet in a fixed tree (warp shuffles, then the eight warps
 //     in order), so equal rows produce bit-identical scores.  HBM-bound:
 //     4*D bytes per row, with a whole row per CTA in flight.
-//  2. topk_select_kernel -- one CTA per sequence (above 8,192 CMEs,
-//     topk_select_cluster_kernel: a cluster of 8, see there).  Scores are mapped to
+//  2. topk_hist_kernel -- one CTA per sequence of up to 32,768 CMEs, when the
+//     call has a workspace for the histogram that the scoring builds (see
+//     there); otherwise topk_select_kernel, one CTA per sequence (above 8,192
+//     CMEs topk_select_cluster_kernel: a cluster of 8).  Scores are mapped to
 //     order-preserving uint32 keys; a 4-pass MSB radix select (8 bits a pass)
 //     finds the key T of the k-th largest score and how many of the keys equal
 //     to T are needed; an ordered compaction then writes the selected indices
@@ -40,10 +43,12 @@ constexpr int kScoreUnroll = 4;
 // costs a little at 1,024).
 constexpr int kSelectThreadsMax = 1024;
 constexpr int kSelectWideN = 8192;
+constexpr int kHistTop = 2048;  // bins of the top 11 bits of a key
 
-__global__ void __launch_bounds__(kScoreThreads)
+__global__ void __launch_bounds__(kScoreThreads, 2048 / kScoreThreads)
 cosine_scores_kernel(const float* __restrict__ qv, const float* __restrict__ bank, int N, int D,
-                     long long rows, float* __restrict__ scores, float* __restrict__ sqnorm) {
+                     long long rows, float* __restrict__ scores, float* __restrict__ sqnorm,
+                     unsigned int* __restrict__ hist) {
   constexpr int kWarpsPerCta = kScoreThreads / 32;
   __shared__ float part[3][kWarpsPerCta];
   const int tid = threadIdx.x;
@@ -108,9 +113,74 @@ cosine_scores_kernel(const float* __restrict__ qv, const float* __restrict__ ban
       if (sm > 0.f && sq > 0.f) sc = sd / (sqrtf(sm) * sqrtf(sq));
       if (sc == 0.f) sc = 0.f;  // -0 -> +0, so that -0 and +0 tie
       scores[r] = sc;
+      if (hist) atomicAdd(hist + b * kHistTop + (orderable(sc) >> 21), 1u);  // see topk_hist_kernel
       if (sqnorm) sqnorm[r] = sm;  // for the CME-guided localisation
     }
     __syncthreads();  // part[] is reused by the next row
+  }
+}
+
+// The same scores for rows of up to kWarpScoreD features: a warp takes a row by
+// itself, so there is no barrier, and the 24 warps of an SM keep up to 4 KB each
+// in flight.  A row of 3 to 8 KB is too little for a CTA: most of its time there
+// goes into the two barriers around a load of one or two float4s a thread.
+// Calls back to back, a CTA per row -> a warp per row: 2 x 8,192 CMEs of 768
+// features 31 -> 16 us, 24 x 826 of 1,280 39 -> 26, 16 x 2,000 of 2,048 66 -> 45.  At
+// 4,096 features a CTA per row streams at 6.5 TB/s, and stays.
+constexpr int kWarpScoreD = 2048;
+constexpr int kWarpScoreCtas = 3;   // per SM
+constexpr int kWarpScoreLoads = 8;  // float4s a lane has in flight
+
+__global__ void __launch_bounds__(kScoreThreads, kWarpScoreCtas)
+cosine_scores_warp_kernel(const float* __restrict__ qv, const float* __restrict__ bank, int N, int D,
+                          long long rows, float* __restrict__ scores, float* __restrict__ sqnorm,
+                          unsigned int* __restrict__ hist) {
+  constexpr int U = kWarpScoreLoads;
+  const int lane = threadIdx.x & 31;
+  const int D4 = D >> 2;
+  const long long step = static_cast<long long>(gridDim.x) * (kScoreThreads / 32);
+  pdl_wait();
+  pdl_trigger();
+  for (long long r = static_cast<long long>(blockIdx.x) * (kScoreThreads / 32) + (threadIdx.x >> 5);
+       r < rows; r += step) {
+    const long long b = rows <= 0x7fffffffll
+                            ? static_cast<long long>(static_cast<unsigned>(r) / static_cast<unsigned>(N))
+                            : r / N;
+    const float4* m = reinterpret_cast<const float4*>(bank + r * D);
+    const float4* q = reinterpret_cast<const float4*>(qv + b * D);
+    float dot = 0.f, mm = 0.f, qq = 0.f;
+    for (int i0 = lane; i0 < D4; i0 += 32 * U) {
+      float4 a[U], c[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        a[u] = i0 + 32 * u < D4 ? ld_stream_f4(m + i0 + 32 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        c[u] = i0 + 32 * u < D4 ? __ldg(q + i0 + 32 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        dot = fmaf(a[u].x, c[u].x, dot); dot = fmaf(a[u].y, c[u].y, dot);
+        dot = fmaf(a[u].z, c[u].z, dot); dot = fmaf(a[u].w, c[u].w, dot);
+        mm = fmaf(a[u].x, a[u].x, mm); mm = fmaf(a[u].y, a[u].y, mm);
+        mm = fmaf(a[u].z, a[u].z, mm); mm = fmaf(a[u].w, a[u].w, mm);
+        qq = fmaf(c[u].x, c[u].x, qq); qq = fmaf(c[u].y, c[u].y, qq);
+        qq = fmaf(c[u].z, c[u].z, qq); qq = fmaf(c[u].w, c[u].w, qq);
+      }
+    }
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) {
+      dot += __shfl_xor_sync(0xffffffffu, dot, off);
+      mm += __shfl_xor_sync(0xffffffffu, mm, off);
+      qq += __shfl_xor_sync(0xffffffffu, qq, off);
+    }
+    if (lane == 0) {
+      float sc = 0.f;
+      if (mm > 0.f && qq > 0.f) sc = dot / (sqrtf(mm) * sqrtf(qq));
+      if (sc == 0.f) sc = 0.f;  // -0 -> +0, so that -0 and +0 tie
+      scores[r] = sc;
+      if (hist) atomicAdd(hist + b * kHistTop + (orderable(sc) >> 21), 1u);  // see topk_hist_kernel
+      if (sqnorm) sqnorm[r] = mm;  // for the CME-guided localisation
+    }
   }
 }
 
@@ -565,7 +635,6 @@ constexpr int kFusedWarps = kFusedThreads / 32;
 constexpr int kFusedRows = 8;                    // rows per CTA at most
 constexpr int kFusedMaxD = 4 * kFusedThreads;    // one float4 per thread and row
 constexpr int kFusedMaxN = 2 * kFusedThreads;    // two keys per thread in the selection
-constexpr int kHistTop = 2048;                   // bins of the top 11 bits of a key
 
 struct FusedArgs {
   const float* qv;        // [B, D], or NULL: pooled from q_tokens
@@ -704,7 +773,7 @@ __device__ __forceinline__ void fused_topk(const uint32_t (&key)[KPT], int N, in
     n_eq += kp == P ? 1u : 0u;
   }
   // the prefixes > P and == P before this thread's, from one prefix sum: both
-  // counts total at most N <= 2048 < 2^16, so the low half never carries
+  // counts total at most N <= 32768 < 2^16, so the low half never carries
   const uint32_t before = fused_scan(n_gt | (n_eq << 16), scan_sel);
   const uint32_t eq_before = before >> 16;
   // the keys > P before this thread's, and the first `need` keys == P
@@ -932,6 +1001,28 @@ score_select_fused_kernel(const __grid_constant__ FusedArgs a) {
   if (last_flag) fused_select(a, b);
 }
 
+// The selection of the two-launch path for banks of up to kHistMaxN CMEs: one
+// CTA of 1,024 threads per sequence, KPT keys a thread, with the search of the
+// one-launch path -- the scoring CTAs have built the histogram of the top 11
+// key bits in the workspace, which leaves two shared-memory levels at most
+// where the radix select of topk_select_kernel takes four passes over the keys.
+// Calls back to back, with topk_select_kernel (above 8,192 CMEs
+// topk_select_cluster_kernel) -> with this one, the CTA-per-row scoring before
+// either: 4 x 1,024 CMEs 21.1 -> 18.0 us, 32 x 2,048 178 -> 165, 1 x 8,192 of 4,096
+// features 46 -> 30, 1 x 4,000 of 1,280 20.3 -> 11.5.  Without a workspace, for k
+// outside 1 .. N - 1 and above kHistMaxN CMEs the others run.
+constexpr int kHistMaxN = 32 * kFusedThreads;
+
+template <int KPT>
+__global__ void __launch_bounds__(kFusedThreads)
+topk_hist_kernel(const __grid_constant__ FusedArgs a, const LocateArgs la) {
+  pdl_wait();  // the scores and the histogram of the kernel before
+  pdl_trigger();
+  const int b = static_cast<int>(blockIdx.x);
+  if (la.sqnorm) locate_window(la, b, a.N);
+  fused_select_impl<KPT>(a, b);
+}
+
 // Rows per CTA of the one-launch path for B sequences of N CMEs of
 // dimension D: the largest R <= kFusedRows dividing N with B N / R CTAs in
 // one wave of one CTA per SM; 0 when there is none (or a limit is exceeded).
@@ -999,12 +1090,38 @@ static int launch_score_select(const float* question_emb, const float* cme_bank,
     return launch_score_select_fused(question_emb, cme_bank, B, N, D, k, idx_out, sc, counters, s,
                                      la, fused_rows);
   const long long rows = static_cast<long long>(B) * N;
-  long long blocks = rows;
-  const long long cap = static_cast<long long>(sm_count()) * (2048 / kScoreThreads);
+  const bool by_warp = D <= kWarpScoreD;
+  constexpr int kWarpsPerCta = kScoreThreads / 32;
+  long long blocks = by_warp ? (rows + kWarpsPerCta - 1) / kWarpsPerCta : rows;
+  const long long cap = static_cast<long long>(sm_count()) * (by_warp ? kWarpScoreCtas : 2048 / kScoreThreads);
   if (blocks > cap) blocks = cap;
-  int st = launch_pdl(cosine_scores_kernel, dim3(static_cast<unsigned>(blocks)), dim3(kScoreThreads),
-                      0, s, question_emb, cme_bank, N, D, rows, sc, la.sqnorm);
+  // the histograms follow the counters in the workspace
+  const bool use_hist = counters && N <= kHistMaxN && k > 0 && k < N;
+  unsigned int* hist = nullptr;
+  if (use_hist)
+    hist = reinterpret_cast<unsigned int*>(reinterpret_cast<char*>(counters) +
+                                           align_up(static_cast<size_t>(B) * sizeof(unsigned int), 256));
+  int st = launch_pdl(by_warp ? cosine_scores_warp_kernel : cosine_scores_kernel,
+                      dim3(static_cast<unsigned>(blocks)), dim3(kScoreThreads), 0, s, question_emb, cme_bank, N, D, rows, sc, la.sqnorm, hist);
   if (st != CMC_OK || (k == 0 && !la.sqnorm)) return st;
+  if (use_hist) {
+    FusedArgs a = {};
+    a.N = N;
+    a.D = D;
+    a.k = k;
+    a.scores = sc;
+    a.counters = counters;
+    a.idx_out = idx_out;
+    a.la = LocateArgs{};  // locate_window serves the localisation here
+    a.hist = hist;
+    const dim3 gd(static_cast<unsigned>(B)), bd(kFusedThreads);
+    if (N <= kFusedThreads) return launch_pdl(topk_hist_kernel<1>, gd, bd, 0, s, a, la);
+    if (N <= 2 * kFusedThreads) return launch_pdl(topk_hist_kernel<2>, gd, bd, 0, s, a, la);
+    if (N <= 4 * kFusedThreads) return launch_pdl(topk_hist_kernel<4>, gd, bd, 0, s, a, la);
+    if (N <= 8 * kFusedThreads) return launch_pdl(topk_hist_kernel<8>, gd, bd, 0, s, a, la);
+    if (N <= 16 * kFusedThreads) return launch_pdl(topk_hist_kernel<16>, gd, bd, 0, s, a, la);
+    return launch_pdl(topk_hist_kernel<32>, gd, bd, 0, s, a, la);
+  }
   static std::once_flag attr_once[64];
   int dev = 0;
   st = record_cuda_error(cudaGetDevice(&dev));

@@ -229,3 +229,26 @@ def test_one_launch_counters_reset_across_calls(cuda_device, name, B):
         torch.cuda.synchronize()
         np.testing.assert_array_equal(idx.cpu().numpy(), si.planted_idx)
         assert not ws[scores_bytes:].cpu().numpy().any(), "counters or histograms left non-zero"
+
+
+@pytest.mark.parametrize("N,D,B", [(1300, 4, 3), (1025, 132, 2), (2049, 2048, 1), (1300, 2052, 1),
+                                   (4096, 132, 2), (4097, 132, 1), (8193, 36, 2), (16384, 132, 1),
+                                   (16385, 36, 2), (32768, 36, 1), (32769, 36, 2)])
+def test_select_two_launches_ties_in_index_order(cuda_device, N, D, B):
+    """Both scoring kernels (rows up to 2,048 features and longer ones) and every size of the
+    selection after them, on two calls that share a workspace.  The rows are unit vectors along
+    an axis and the question holds small whole numbers, so that a score is one of a few dozen
+    values, exact up to one rounding: most of the cut is a tie, which goes to the lower index."""
+    rng = np.random.default_rng(N + D)
+    q = rng.integers(-40, 41, size=(B, D)).astype(np.float32)
+    q[:, 0] = 41.0
+    ws = torch.zeros(cmc.score_select_workspace_size(B, N), dtype=torch.uint8, device=cuda_device)
+    for k in (1, N // 3, N - 1):
+        axis = rng.integers(0, D, size=(B, N))
+        bank = np.zeros((B, N, D), dtype=np.float32)
+        bank[np.arange(B)[:, None], np.arange(N)[None, :], axis] = 1.0
+        got = cmc.score_select(torch.from_numpy(q).to(cuda_device), torch.from_numpy(bank).to(cuda_device),
+                               k, workspace=ws).cpu().numpy()
+        for b in range(B):
+            order = np.lexsort((np.arange(N), -q[b, axis[b]]))
+            np.testing.assert_array_equal(got[b], np.sort(order[:k]), err_msg=f"k={k} b={b}")
