@@ -1508,8 +1508,10 @@ window_append_kernel(uint16_t* __restrict__ ring_k, uint16_t* __restrict__ ring_
 // Tier-1 compaction (the "M*" of Section 2.5, formed once per question):
 //   tier1[b, l, g, i] = bank[b, l, g, idx[b, i]]   for i < k.
 // A CTA copies a block of kGatherRows output rows of one unit: each thread
-// issues all of its 16-byte streaming loads (K and V) before its stores, so a
-// whole block is in flight at once.  Out-of-range indices give a zero row and
+// requests its indices, then issues all of its 16-byte streaming loads (K and
+// V), then stores, so a whole block is in flight at once (an index loaded
+// just before its row made four trips of the indices: prologue and compaction of
+// four requests 80.8 us, now 76.2).  Out-of-range indices give a zero row and
 // CMC_DEVFLAG_BAD_INDEX.
 constexpr int kGatherRows = 64;
 constexpr int kGatherThreads = 256;
@@ -1537,20 +1539,22 @@ tier1_gather_kernel(const uint4* __restrict__ bank_k, const uint4* __restrict__ 
     const int i0 = static_cast<int>(blk - u * row_blocks) * kGatherRows;
     const int32_t* irow = idx + (u / LH) * k;
     uint4 kv[kPer], vv[kPer];
+    int row[kPer];
+#pragma unroll
+    for (int e = 0; e < kPer; ++e) {
+      const int i = i0 + (threadIdx.x + e * kGatherThreads) / CPR;
+      row[e] = i < k ? __ldg(irow + i) : 0;
+    }
 #pragma unroll
     for (int e = 0; e < kPer; ++e) {
       const int x = threadIdx.x + e * kGatherThreads;
-      const int i = i0 + x / CPR;
+      const bool in = static_cast<unsigned>(row[e]) < static_cast<unsigned>(N);
+      bad |= !in;  // past k the row is 0, and N >= 1
       kv[e] = vv[e] = make_uint4(0u, 0u, 0u, 0u);
-      if (i < k) {
-        const int j = __ldg(irow + i);
-        if (static_cast<unsigned>(j) < static_cast<unsigned>(N)) {
-          const long long src = (u * N + j) * CPR + x % CPR;
-          kv[e] = ld_stream(bank_k + src);
-          vv[e] = ld_stream(bank_v + src);
-        } else {
-          bad = true;
-        }
+      if (i0 + x / CPR < k && in) {
+        const long long src = (u * N + row[e]) * CPR + x % CPR;
+        kv[e] = ld_stream(bank_k + src);
+        vv[e] = ld_stream(bank_v + src);
       }
     }
 #pragma unroll
