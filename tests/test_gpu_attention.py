@@ -784,3 +784,25 @@ def test_window_append_one_cta_and_clusters(cuda_device, L, Hkv, d):
                 ring[which][b, :, :, p % W] = new[which][b]
             assert torch.equal(dev_ring[which][b].cpu(), ring[which][b]), (b, which)
     assert pos.cpu().tolist() == [p + 1 if p >= 0 else p for p in pos0]
+
+
+@pytest.mark.parametrize("per_tile", [3.0, 7.9, 8.1, 40.0, -7.9])
+@pytest.mark.parametrize("d", [64, 128])
+def test_logits_rising_from_tile_to_tile(cuda_device, d, per_tile):
+    """The exponentials' reference moves only when a tile's largest logit exceeds it by more than
+    8 (in powers of two): logits that rise, or fall, by around that much from tile to tile."""
+    W = 640
+    w = WORKLOADS["tiny"].with_(name="rising", d=d, N=64, k=0, W=W, T=2)
+    P = Problem(w, cuda_device)
+    st = step_inputs(w, 0)
+    slope = per_tile / 64 * np.log(2.0)  # of the natural logits, a key
+    keys = np.zeros((w.B, w.L, w.Hkv, W, d), dtype=np.float32)
+    keys[..., 0] = slope * np.arange(W) + 0.01 * np.random.default_rng(1).standard_normal(W)
+    bits = host_bits(torch.from_numpy(keys).to(torch.bfloat16))
+    P.ring_k.copy_(dev_bf16(bits, cuda_device))
+    P.o_ring_k[:] = bits
+    q = np.zeros((w.B, w.L, w.Hq, d), dtype=np.float32)
+    q[..., 0] = np.linspace(0.5, 1.0, w.Hq)
+    st.q[:] = host_bits(torch.from_numpy(q).to(torch.bfloat16))
+    out, ref = P.step(st, scale=1.0)
+    assert_attn_close(to_f64(out), ref, f"{per_tile} a tile")
