@@ -1651,17 +1651,15 @@ static bool encode_rows(CUtensorMap* map, const void* base, long long rows, int 
 // Pipeline depth: stages of 64 keys per CTA.  Three stages keep a CTA at
 // ~110 KB of shared memory at d = 128, G <= 4, so two CTAs share an SM.
 constexpr int kStages = 3;
-// Box tiles per CTA prefetched into L2 before the grid dependency wait.  With
-// the streamed K/V loads marked evict-first, five tiles (160 KB per CTA, some
-// in free slots while the previous launch runs, most in its tail) measured
-// best at the Llama-3-8B shape (14.20 us against 14.34 for four, 14.30 for six,
-// 14.7 for three or eight); without the evict-first policy one tile was best.
-// A rolling prefetch a few tiles ahead of the TMA issue, on top, was slower at
-// every distance (16.2-16.9 us).  That is for one stream of launches: with
-// independent requests' launches on four streams, whose launches already run
-// through each other's edges, no prefetch measured best (11.92 us against
-// 12.11 for one tile, 12.32 for two, 12.89 for five), so the depth is a
-// setting (cmc_set_l2_prefetch_tiles) with this default.
+// Box tiles per CTA prefetched into L2 before the grid dependency wait, at most
+// (see prefetch_cap).  The streamed K/V loads are marked evict-first; without
+// that policy one tile was best.  A rolling prefetch a few tiles ahead of the
+// TMA issue, on top, was slower at every distance (16.2-16.9 against 14.2 us a
+// step).  That is for one stream of launches: with independent requests'
+// launches on four streams, whose launches already run through each other's
+// edges, no prefetch measured best (11.92 us against 12.11 for one tile, 12.32
+// for two, 12.89 for five), so the depth is a setting
+// (cmc_set_l2_prefetch_tiles) with this default.
 constexpr int kL2PrefetchTiles = 5;
 constexpr int kMaxL2PrefetchTiles = 64;
 static std::atomic<int> g_l2_prefetch_tiles{kL2PrefetchTiles};
@@ -1752,6 +1750,24 @@ static int plan_attn(long long total_tiles, int tpu, AttnPlan* pl) {
   return CMC_OK;
 }
 
+// The most tiles a CTA of a plan gains from prefetching (of the setting's).  us a
+// round at depth 1 / 2 / 3 / 5, two requests in turn on one stream:
+//   clusters:     16 x (64 + 512 keys) 67.5 / 68.2 / 69.3 / 71.4, the same as
+//                 separate append and attention 42.0 / 43.8 / 47.1 / 50.1, 12 x
+//                 (200 + 900) 97.6 / 97.2 / 99.4 / 104.1, 16 x (256 + 2,048) 49
+//                 at each: a CTA's share is a few tiles, which it is about to
+//                 load itself;
+//   whole units:  32 layers x (128 + 512) 58.6 / 57.1 / 56.8 / 57.2 (56.5 at 4), 32
+//                 layers of 8 x (30 + 130) 38.2 at 2 and 37.0 at 4 and 5; at
+//                 d = 64, with half the bytes a tile, 504 units 23.6 / 23.5 / 23.6
+//                 / 24.4;
+//   split units:  320 units 44.1 / 44.5 / 44.7 / 43.5.
+static int prefetch_cap(const AttnPlan& pl, int d) {
+  if (pl.cm > 0) return 2;
+  if (pl.split) return kMaxL2PrefetchTiles;
+  return d == 64 ? 2 : 4;
+}
+
 // Launches the attention kernel with programmatic stream serialization and,
 // for a cluster plan, the cluster dimension.
 template <int D, int G, bool FUSED, bool ROPE>
@@ -1789,6 +1805,7 @@ static int launch_attn(const AttnMaps& maps, const AttnParams& p0, long long tot
   p.base = static_cast<int>(pl.base);
   p.rem = static_cast<int>(pl.rem);
   p.cm = pl.cm;
+  p.l2_prefetch = p0.l2_prefetch < prefetch_cap(pl, D) ? p0.l2_prefetch : prefetch_cap(pl, D);
   p.slice = pl.cm > 0 ? (G * D / 4 + pl.cm - 1) / pl.cm : 0;
   if (p.idx) {
     // Gathered Tier-1: each CTA begins with a pipeline's depth of ring tiles,
