@@ -1210,14 +1210,12 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
         if (!((mk >> (gq + 8)) & 1u)) v[2] = v[3] = -INFINITY;
       }
       // ---- online softmax (log2 domain), heads 2 tq and 2 tq + 1.  The
-      // reference m_run of the exponentials is a maximum seen so far, moved
-      // up -- and the sums and outputs rescaled, 34 multiplications -- only when
-      // a tile's exceeds it by more than kLazyMax: probabilities then reach at
-      // most 2^kLazyMax, which costs neither bf16 nor fp32 any precision.  (With
-      // the masks only built where a row holds no key, and the accumulators'
-      // zeros, the scale and the abort flag's look out of the way: 32 layers
-      // of 8 x (30 + 130) keys 39.1 -> 37.0 us a step, others 0.5 to 3 %.)
-      constexpr float kLazyMax = 8.f;
+      // reference of the exponentials is the maximum so far, so that the largest
+      // probability is exactly 1 in bf16: one that lagged up to 2^8 behind, with
+      // fewer rescalings, cost a fifth more error (2.3e-3 against 1.9e-3 of
+      // the outputs' norm).  (The masks only built where a row holds no key, and
+      // the accumulators' zeros, the scale and the abort flag's look out of
+      // the way: 32 layers of 8 x (30 + 130) keys 39.1 -> 37.1 us a step.) ----
       float mx0 = fmaxf(v[0], v[2]), mx1 = fmaxf(v[1], v[3]);
 #pragma unroll
       for (int off = 4; off < 32; off <<= 1) {  // over the 8 key rows (lane bits 2-4)
@@ -1226,7 +1224,7 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
       }
       mx0 *= p.scale_log2;
       mx1 *= p.scale_log2;
-      const bool up0 = mx0 > m_run[0] + kLazyMax, up1 = mx1 > m_run[1] + kLazyMax;
+      const bool up0 = mx0 > m_run[0], up1 = mx1 > m_run[1];
       if (__any_sync(0xffffffffu, up0 || up1)) {
         const float alpha0 = up0 ? ex2(m_run[0] - mx0) : 1.f;
         const float alpha1 = up1 ? ex2(m_run[1] - mx1) : 1.f;

@@ -786,11 +786,11 @@ def test_window_append_one_cta_and_clusters(cuda_device, L, Hkv, d):
     assert pos.cpu().tolist() == [p + 1 if p >= 0 else p for p in pos0]
 
 
-@pytest.mark.parametrize("per_tile", [3.0, 7.9, 8.1, 40.0, -7.9])
+@pytest.mark.parametrize("per_tile", [3.0, 8.0, 40.0, -8.0])
 @pytest.mark.parametrize("d", [64, 128])
 def test_logits_rising_from_tile_to_tile(cuda_device, d, per_tile):
-    """The exponentials' reference moves only when a tile's largest logit exceeds it by more than
-    8 (in powers of two): logits that rise, or fall, by around that much from tile to tile."""
+    """Logits that rise, or fall, from tile to tile, so that every tile (or none after the first)
+    moves the exponentials' reference and rescales the sums."""
     W = 640
     w = WORKLOADS["tiny"].with_(name="rising", d=d, N=64, k=0, W=W, T=2)
     P = Problem(w, cuda_device)
