@@ -181,20 +181,34 @@ denoise_pass_kernel(const float* __restrict__ emb, const int32_t* __restrict__ n
   __shared__ uint32_t nib[kPassThreads / 32];        // each warp's four pass bits
   __shared__ int wmax[kPassThreads / 32], wsum[kPassThreads / 32];  // the fused compaction's scans
   __shared__ int last_flag;
-  pdl_wait();
-  pdl_trigger();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nchunks = (H + kPassChunk - 1) / kPassChunk;
   const uint32_t sbase = static_cast<uint32_t>(__cvta_generic_to_shared(dn_stage));
   const int r0 = warp * TPW;  // this warp's first token row in the tile
+  // The context and the first token of a tile: a CTA's first before the grid
+  // dependency wait, in 32 bits where the tile numbers fit.  With the -1s
+  // written after the first chunks are requested, 1 to 2 % of a call (4 contexts of
+  // 4,096 tokens 22.5 -> 22.0 us, 8 of 8,000 50.8 -> 50.0).
+  int b, i0;
+  auto place = [&](long long t) {
+    if (tiles <= 0x7fffffffll)
+      b = static_cast<int>(static_cast<unsigned>(t) / static_cast<unsigned>(tiles_per_ctx));
+    else
+      b = static_cast<int>(t / tiles_per_ctx);
+    i0 = static_cast<int>(t - static_cast<long long>(b) * tiles_per_ctx) * kPassTile;
+  };
+  place(blockIdx.x);
+  pdl_wait();
+  pdl_trigger();
   for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-    const int b = static_cast<int>(tile / tiles_per_ctx);
-    const int i0 = static_cast<int>(tile - static_cast<long long>(b) * tiles_per_ctx) * kPassTile;
+    if (tile != blockIdx.x) place(tile);
     int n = n_tokens ? n_tokens[b] : n_max;
     n = n < 0 ? 0 : (n > n_max ? n_max : n);
     uint8_t* pb = pass + static_cast<long long>(b) * n_max;
     // the compaction overwrites the kept positions; everything else stays -1
-    if (tid < kPassTile && i0 + tid < n_max) kept_idx[static_cast<long long>(b) * n_max + i0 + tid] = -1;
+    auto clear_kept = [&]() {
+      if (tid < kPassTile && i0 + tid < n_max) kept_idx[static_cast<long long>(b) * n_max + i0 + tid] = -1;
+    };
     // Thread 0 writes the tile's pass word (after the barrier that makes the
     // warps' bits and every thread's writes precede it) and, fused, adds the
     // tile to the context's count with an acq_rel atomic (releasing this CTA's
@@ -229,6 +243,7 @@ denoise_pass_kernel(const float* __restrict__ emb, const int32_t* __restrict__ n
       }
     };
     if (i0 >= n) {  // a tile past the context's tokens: flags 0
+      clear_kept();
       if (tid < kPassTile && i0 + tid < n_max) pb[i0 + tid] = 0;
       tile_done(true);
       continue;
@@ -262,6 +277,7 @@ denoise_pass_kernel(const float* __restrict__ emb, const int32_t* __restrict__ n
       if (c < nchunks) issue(c);
       dn_commit();
     }
+    clear_kept();
     // v: the norms of rows r0 .. r0+TPW+G-1, then dot(t, s) at TPW + G + t G + s
     float v[NV16];
 #pragma unroll
