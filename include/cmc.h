@@ -112,7 +112,10 @@ CMC_API size_t cmc_denoise_workspace_size(int B, int n_max);
  *   workspace   >= cmc_denoise_workspace_size(B, n_max) bytes, zero-filled
  *               before its first use: its last bytes hold one completion
  *               counter per context, which every call leaves zero (calls
- *               that share a workspace must be ordered, e.g. one stream);
+ *               that share a workspace must be ordered, e.g. one stream).
+ *               Where the counters lie depends on B and n_max, so a
+ *               workspace serves one (B, n_max): zero-fill it again before
+ *               a call of another shape, even one of the same size;
  *               on completion its first B * n_max bytes hold each token's
  *               threshold-test result (1 passed, 0 not or past n_tokens)
  *
@@ -174,9 +177,12 @@ CMC_API size_t cmc_score_select_workspace_size(int B, int N);
  *                 aligned, ZERO-FILLED ONCE before its first use: it holds
  *                 one completion counter and one histogram of the scores'
  *                 top 11 key bits per sequence, which every call leaves at
- *                 zero again (the scores part may hold anything).  Calls that
- *                 share a workspace must be ordered (e.g. one stream).  It may
- *                 be NULL when scores_out is given.
+ *                 zero again (the scores part may hold anything).  Where they
+ *                 lie depends on B and N, so a workspace serves one (B, N):
+ *                 zero-fill it again before a call of another shape, even one
+ *                 of the same size.  Calls that share a workspace must be
+ *                 ordered (e.g. one stream).  It may be NULL when scores_out
+ *                 is given.
  *
  * Small banks with a workspace (D <= 4096, N <= 2048, and B * N rows that
  * CTAs of at most 8 rows of one sequence cover in one wave of one CTA per SM)
@@ -225,7 +231,8 @@ CMC_API size_t cmc_question_select_workspace_size(int B, int N);
  *   alpha_out, start_out  int32 [B]; either may be NULL; when both are NULL
  *                    chunk_offset, ctx_len and W are not used
  *   workspace        >= cmc_question_select_workspace_size(B, N) bytes,
- *                    16-byte aligned, zero-filled once before its first use
+ *                    16-byte aligned, zero-filled once before its first use,
+ *                    for one (B, N)
  *                    (as for cmc_score_select: scores, squared norms, then
  *                    B completion counters, B histograms of 2,048 counts and
  *                    B 64-bit argmax slots, all left at zero by every call)

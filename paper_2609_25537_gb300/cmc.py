@@ -118,7 +118,8 @@ def denoise(emb: torch.Tensor, *, n_tokens: Optional[torch.Tensor] = None, g: in
     """Positions of the tokens kept by the graph-based denoising, int32
     [B, n_max] ascending then -1, and their counts int32 [B]; see
     cmc_denoise.  Defaults: the paper's g = 3, tau = 0.05, keep-minimum 16.
-    A given ``workspace`` must have been zero-filled before its first use."""
+    A given ``workspace`` must have been zero-filled before its first use and
+    serves one (B, n_max)."""
     _need(emb, "emb", torch.float32, 3)
     dev = emb.device
     B, n_max, H = emb.shape
@@ -129,7 +130,7 @@ def denoise(emb: torch.Tensor, *, n_tokens: Optional[torch.Tensor] = None, g: in
     kept = torch.empty((B, n_max), dtype=torch.int32, device=dev)
     count = torch.empty(B, dtype=torch.int32, device=dev)
     if workspace is None:
-        workspace = _counter_workspace("denoise", int(lib().cmc_denoise_workspace_size(B, n_max)), dev)
+        workspace = _counter_workspace("denoise", B, n_max, dev)
     st = lib().cmc_denoise(_p(emb), _p(n_tokens), B, n_max, H, g, float(tau), keep_every,
                            _p(kept), _p(count), _p(workspace),
                            workspace.numel() * workspace.element_size(), _stream(dev))
@@ -178,13 +179,19 @@ def score_select_workspace_size(B: int, N: int) -> int:
 _counter_ws_cache: Dict[Tuple, torch.Tensor] = {}
 
 
-def _counter_workspace(kind: str, nbytes: int, device: torch.device) -> torch.Tensor:
-    """A zero-filled workspace, one per (kind, device, stream, size): its
-    completion counters start at zero, and every call leaves them so."""
-    key = (kind, device.index, _stream(device), nbytes)
+def _counter_workspace(kind: str, B: int, n: int, device: torch.device) -> torch.Tensor:
+    """A zero-filled workspace, one per (kind, device, stream, B, n): its
+    counters and histograms start at zero, and every call leaves them so.
+    Where they lie depends on the shape, and shapes of one size exist (B = 1,
+    4,096 CMEs and B = 2, 1,024), so the size alone is no key: the one's
+    scores would be the other's histograms."""
+    key = (kind, device.index, _stream(device), B, n)
     ws = _counter_ws_cache.get(key)
     if ws is None:
-        ws = torch.zeros(nbytes, dtype=torch.uint8, device=device)
+        size = {"denoise": lib().cmc_denoise_workspace_size,
+                "select": lib().cmc_score_select_workspace_size,
+                "question": lib().cmc_question_select_workspace_size}[kind]
+        ws = torch.zeros(int(size(B, n)), dtype=torch.uint8, device=device)
         _counter_ws_cache[key] = ws
     return ws
 
@@ -196,7 +203,8 @@ def score_select(question_emb: torch.Tensor, cme_bank: torch.Tensor, k: int, *,
                  workspace: Optional[torch.Tensor] = None) -> torch.Tensor:
     """Top-k CMEs by cosine similarity to the question vector, as int32 [B, k]
     indices in ascending (document) order.  See cmc_score_select.  A given
-    ``workspace`` must have been zero-filled before its first use."""
+    ``workspace`` must have been zero-filled before its first use and serves
+    one (B, N)."""
     _need(cme_bank, "cme_bank", torch.float32, 3)
     dev = cme_bank.device
     _need(question_emb, "question_emb", torch.float32, 2, dev)
@@ -213,7 +221,7 @@ def score_select(question_emb: torch.Tensor, cme_bank: torch.Tensor, k: int, *,
         if tuple(scores_out.shape) != (B, N):
             raise ValueError(f"scores_out shape {tuple(scores_out.shape)} != {(B, N)}")
     if workspace is None:
-        workspace = _counter_workspace("select", score_select_workspace_size(B, N), dev)
+        workspace = _counter_workspace("select", B, N, dev)
     ws_bytes = workspace.numel() * workspace.element_size()
     st = lib().cmc_score_select(_p(question_emb), _p(cme_bank), B, N, D, k, _p(idx_out),
                                 _p(scores_out), _p(workspace), ws_bytes, _stream(dev))
@@ -230,7 +238,8 @@ def question_select(question_tokens: torch.Tensor, cme_bank: torch.Tensor, k: in
     """The question-side prologue; see cmc_question_select.  Returns
     (q_vec fp32 [B, D], idx int32 [B, k], alpha int32 [B] or None,
     start int32 [B] or None); alpha and start when chunk_offset, ctx_len
-    and W are given."""
+    and W are given.  A given ``workspace`` must have been zero-filled before
+    its first use and serves one (B, N)."""
     _need(cme_bank, "cme_bank", torch.float32, 3)
     dev = cme_bank.device
     _need(question_tokens, "question_tokens", torch.float32, 3, dev)
@@ -253,8 +262,7 @@ def question_select(question_tokens: torch.Tensor, cme_bank: torch.Tensor, k: in
     alpha = torch.empty(B, dtype=torch.int32, device=dev) if locate else None
     start = torch.empty(B, dtype=torch.int32, device=dev) if locate else None
     if workspace is None:
-        workspace = _counter_workspace(
-            "question", int(lib().cmc_question_select_workspace_size(B, N)), dev)
+        workspace = _counter_workspace("question", B, N, dev)
     st = lib().cmc_question_select(
         _p(question_tokens), _p(q_len), Lq, _p(cme_bank), B, N, D, k, _p(chunk_offset),
         _p(ctx_len), int(W or 0), _p(q_vec), _p(idx), _p(alpha), _p(start), _p(workspace),

@@ -109,3 +109,18 @@ def test_denoise_one_launch_and_two_launch_paths(cuda_device):
             _check(emb, n_tok, 3, 0.3, 16, cuda_device, whole=rep == 0, ws=ws)
             tail = ws[-256:].cpu().numpy()
             assert not tail.any(), "completion counters not left at zero"
+
+
+def test_kept_workspaces_of_two_shapes_of_one_size(cuda_device):
+    """Two shapes in turn on one stream, on the workspaces that the binding keeps: of one size,
+    with the second's completion counters where the first's pass words lie."""
+    size = cmc.lib().cmc_denoise_workspace_size
+    assert size(2, 1600) == size(65, 32)
+    rng = np.random.default_rng(8)
+    with torch.cuda.stream(torch.cuda.Stream(cuda_device)):
+        for B, n in ((2, 1600), (65, 32)):
+            emb = np.cumsum(rng.standard_normal((B, n, 32)), axis=1).astype(np.float32)
+            kept, cnt = cmc.denoise(torch.from_numpy(emb).to(cuda_device), tau=-2.0)  # all but the last
+            assert cnt.cpu().tolist() == [n - 1] * B
+            want = np.append(np.arange(n - 1), -1)
+            assert (kept.cpu().numpy() == want).all()

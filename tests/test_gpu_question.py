@@ -111,3 +111,21 @@ def test_question_prologue_ties_inside_a_cta_and_workspace_reuse(cuda_device):
         np.testing.assert_array_equal(start.cpu().numpy(), rstart)
         tail = ws[2 * (-(-B * N * 4 // 256) * 256):].cpu().numpy()
         assert not tail.any(), "counters, histograms or argmax slots not left at zero"
+
+
+@pytest.mark.parametrize("first,second", [((1, 3072), (2, 1024)), ((1, 5120), (2, 2048)),
+                                          ((2, 2048), (4, 512))])
+def test_kept_workspaces_of_two_shapes_of_one_size(cuda_device, first, second):
+    """Two shapes in turn on one stream, on the workspaces that the binding keeps: of one size,
+    with the histograms elsewhere."""
+    size = cmc.lib().cmc_question_select_workspace_size
+    assert size(*first) == size(*second)
+    with torch.cuda.stream(torch.cuda.Stream(cuda_device)):
+        for B, N in (first, second, first, second):
+            rng = np.random.default_rng([B, N])
+            tokens = rng.standard_normal((B, 5, 64)).astype(np.float32)
+            bank = rng.standard_normal((B, N, 64)).astype(np.float32)
+            bank[:, N // 3] *= 2.0  # the largest norm
+            _norm_gap_ok(bank)
+            offs = np.tile(np.arange(N, dtype=np.int32) * 4, (B, 1))
+            _check(tokens, None, bank, N // 8, offs, np.full(B, 4 * N, dtype=np.int32), 64, cuda_device)

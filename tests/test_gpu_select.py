@@ -252,3 +252,24 @@ def test_select_two_launches_ties_in_index_order(cuda_device, N, D, B):
         for b in range(B):
             order = np.lexsort((np.arange(N), -q[b, axis[b]]))
             np.testing.assert_array_equal(got[b], np.sort(order[:k]), err_msg=f"k={k} b={b}")
+
+
+# Shapes of one workspace size whose histograms lie elsewhere: the scores of the first call of
+# a pair cover histograms of the second.
+SAME_SIZE = [((1, 4096), (2, 1024)), ((1, 6144), (2, 2048)), ((2, 4096), (4, 1024)),
+             ((4, 4096), (8, 1024)), ((1, 2112), (2, 32))]
+
+
+@pytest.mark.parametrize("first,second", SAME_SIZE)
+def test_kept_workspaces_of_two_shapes_of_one_size(cuda_device, first, second):
+    """Two shapes in turn on one stream, on the workspaces that the binding keeps."""
+    assert cmc.score_select_workspace_size(*first) == cmc.score_select_workspace_size(*second)
+    with torch.cuda.stream(torch.cuda.Stream(cuda_device)):
+        for B, N in (first, second, first, second):
+            rng = np.random.default_rng(B * N)
+            q = rng.standard_normal((B, 64)).astype(np.float32)
+            bank = rng.standard_normal((B, N, 64)).astype(np.float32)
+            k = max(1, N // 8)
+            idx = cmc.score_select(dev_f32(q, cuda_device), dev_f32(bank, cuda_device), k)
+            ref, _ = oracle.score_select(q, bank, k)
+            np.testing.assert_array_equal(idx.cpu().numpy(), ref)
