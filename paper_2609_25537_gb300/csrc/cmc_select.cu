@@ -649,7 +649,8 @@ struct FusedArgs {
   unsigned int* counters; // [B]: zero before the call, zero after it
   int32_t* idx_out;       // [B, k]
   LocateArgs la;          // la.sqnorm: also write squared norms and localise
-  unsigned int* hist;     // [B, kHistTop]: counts of the scores' top 11 key bits (zero before, zero after)
+  unsigned int* hist;     // [B, kHistTop]: counts of the scores' top 11 key bits (zero before,
+                          // zero after; left alone for k = 0 and k = N)
 };
 
 // Exclusive prefix sum over the block of one value per thread (warps in
@@ -964,7 +965,9 @@ score_select_fused_kernel(const __grid_constant__ FusedArgs a) {
       if (sm > 0.f && qq > 0.f) sc = sd / (sqrtf(sm) * sqrtf(qq));
       if (sc == 0.f) sc = 0.f;  // -0 -> +0, so that -0 and +0 tie
       a.scores[r0 + warp] = sc;
-      atomicAdd(a.hist + static_cast<long long>(b) * kHistTop + (orderable(sc) >> 21), 1u);
+      // only for a search, which puts the counts back to zero
+      if (a.k > 0 && a.k < a.N)
+        atomicAdd(a.hist + static_cast<long long>(b) * kHistTop + (orderable(sc) >> 21), 1u);
       if (a.la.sqnorm) a.la.sqnorm[r0 + warp] = sm;
       rsq_s[warp] = sm;
     }

@@ -273,3 +273,19 @@ def test_kept_workspaces_of_two_shapes_of_one_size(cuda_device, first, second):
             idx = cmc.score_select(dev_f32(q, cuda_device), dev_f32(bank, cuda_device), k)
             ref, _ = oracle.score_select(q, bank, k)
             np.testing.assert_array_equal(idx.cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("N,B", [(1024, 1), (1216, 1), (256, 3), (4096, 2)])
+def test_calls_that_need_no_search_leave_the_histograms_at_zero(cuda_device, N, B):
+    """k = N and k = 0 select without the histogram search; a real k after them, on the same
+    workspace, must not meet their counts (one launch for the first three banks)."""
+    w = WORKLOADS["tiny"].with_(name="search", B=B, N=N, D=64, k=N // 8)
+    si = selection_inputs(w)
+    qd, bd = dev_f32(si.question_emb, cuda_device), dev_f32(si.cme_bank, cuda_device)
+    ws = torch.zeros(cmc.score_select_workspace_size(B, N), dtype=torch.uint8, device=cuda_device)
+    scores_bytes = -(-B * N * 4 // 256) * 256
+    for k in (N, 0, w.k, N, 0, 0, w.k):
+        idx = cmc.score_select(qd, bd, k, workspace=ws).cpu().numpy()
+        np.testing.assert_array_equal(idx, si.planted_idx if 0 < k < N
+                                      else np.tile(np.arange(k), (B, 1)))
+        assert not ws[scores_bytes:].cpu().numpy().any(), "counters or histograms left non-zero"
