@@ -1092,7 +1092,10 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
       mk = static_cast<uint32_t>(keys >> (16 * warp)) & 0xFFFFu;
     }
     if (dead) mk = 0u;
-    bool wrote_stage = false;  // generic-proxy writes into the stage by this warp
+    // generic-proxy writes into the stage: by this warp below, or a gathered
+    // tile's rows (the producer's cp.async copies; the full barrier orders them
+    // before this warp)
+    bool wrote_stage = gathered_tile(p, cc);
 
     if (FUSED && new_row >= 0 && (new_row >> 4) == warp) {
       // Patch the new token over its stale ring row (swizzled) and append it

@@ -806,3 +806,21 @@ def test_logits_rising_from_tile_to_tile(cuda_device, d, per_tile):
     st.q[:] = host_bits(torch.from_numpy(q).to(torch.bfloat16))
     out, ref = P.step(st, scale=1.0)
     assert_attn_close(to_f64(out), ref, f"{per_tile} a tile")
+
+
+@pytest.mark.parametrize("B,d", [(1, 128), (38, 128), (40, 128), (80, 64)])
+def test_gathered_tiles_between_ring_tiles_repeat_exactly(cuda_device, B, d):
+    """Three gathered Tier-1 tiles between the ring tiles of a unit, so that a stage changes from
+    gathered rows to boxes: clusters, one unit a CTA, and units cut between CTAs.  A read-only
+    call on one state gives the same bits each time, near the oracle's."""
+    w = _cluster_case(B, 1, 8, 130, 704 if B == 1 else 448, N=300, T=1, d=d)
+    P = Problem(w, cuda_device, mode="gather")
+    q = step_inputs(w, 0).q
+    args = (dev_bf16(q, cuda_device), P.t1k, P.t1v, P.idx, P.ring_k, P.ring_v, P.pos)
+    first = cmc.two_tier_decode_attn(*args, workspace=P.ws)
+    ref = oracle.two_tier_attention(q, P.kv.tier1_k, P.kv.tier1_v, P.idx_host, P.o_ring_k,
+                                    P.o_ring_v, P.o_pos)
+    assert_attn_close(to_f64(first), ref, f"B={B} d={d}")
+    for _ in range(50):
+        assert torch.equal(cmc.two_tier_decode_attn(*args, workspace=P.ws), first)
+    assert P.ws.status() == 0
