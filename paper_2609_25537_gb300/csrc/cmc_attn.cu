@@ -1901,7 +1901,11 @@ static void rope_turns_table(double theta, int d, unsigned long long (&out)[64])
 // The slot of g_rope_tables holding the table of (theta, d) on the current
 // device, writing it on first use; -1 (use the kernel parameters) when the
 // slots are full, the stream is being captured into a graph, or the copy
-// fails.  The copy is synchronous, so every later launch sees the table.
+// fails.  A copy from pageable memory may return before it has reached the
+// device, and is ordered with the legacy default stream only, while the kernel
+// reads the table on any stream, before its grid dependency wait: so the slot
+// is used once that stream has been waited for, and every later launch sees
+// the table.
 struct RopeSlots {
   std::mutex mu;
   int n = 0;
@@ -1928,7 +1932,8 @@ static int rope_slot(double theta, int d, const unsigned long long* table, cudaS
   }
   if (cudaMemcpyToSymbol(g_rope_tables, table, 64 * sizeof(unsigned long long),
                          static_cast<size_t>(c.n) * 64 * sizeof(unsigned long long),
-                         cudaMemcpyHostToDevice) != cudaSuccess) {
+                         cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {
     cudaGetLastError();
     return -1;
   }

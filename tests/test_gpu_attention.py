@@ -708,6 +708,31 @@ def test_rope_frequency_table_in_device_memory_or_parameters(cuda_device):
     assert_attn_close(to_f64(out_b), ref, "rope table paths")
 
 
+@pytest.mark.parametrize("theta", [34567.891, 45678.912])  # used by no other test
+def test_rope_first_use_on_a_side_stream(cuda_device, theta):
+    """The first step of a theta on a stream that is not ordered with the default one, beside work
+    there: its table must have arrived before the launch reads it."""
+    w = WORKLOADS["tiny"].with_(B=2, T=1)
+    st = step_inputs(w, 0)
+    q, kn, vn = (dev_bf16(x, cuda_device) for x in (st.q, st.k_new, st.v_new))
+    big = torch.empty(1 << 28, dtype=torch.uint8, device=cuda_device)
+    outs, rings = [], []
+    for _ in range(2):
+        P = Problem(w, cuda_device, mode="dense")
+        torch.cuda.synchronize()
+        for _ in range(8):
+            big.zero_()
+        with torch.cuda.stream(torch.cuda.Stream(cuda_device)):
+            outs.append(cmc.decode_step(q, P.t1k, P.t1v, P.idx, P.ring_k, P.ring_v, P.pos, kn, vn,
+                                        workspace=P.ws, rope_theta=theta, rope_offset=w.k))
+        torch.cuda.synchronize()
+        rings.append(P.ring_k)
+    assert torch.equal(outs[0], outs[1]) and torch.equal(rings[0], rings[1])
+    ref = oracle.decode_step_rope(st.q, P.kv.tier1_k, P.kv.tier1_v, P.idx_host, P.o_ring_k, P.o_ring_v,
+                                  P.o_pos, st.k_new, st.v_new, theta=theta, rope_offset=w.k)
+    assert_attn_close(to_f64(outs[0]), ref, "first use")
+
+
 def test_rope_many_thetas(cuda_device):
     """More distinct thetas than device table slots: the later ones use the
     kernel parameters; every step matches the oracle."""
