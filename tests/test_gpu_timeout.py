@@ -86,3 +86,47 @@ def test_stalled_waits_time_out_and_context_survives(cuda_device, name, dense, r
     assert_attn_close(to_f64(out), ref, f"{name} after the stalled call")
     assert ws.status() == 0
     np.testing.assert_array_equal(pos.cpu().numpy(), o_pos)
+
+
+@pytest.mark.parametrize("rope", [False, True])
+@pytest.mark.parametrize("gather", [False, True])
+def test_stalled_call_leaves_other_ring_rows_alone(cuda_device, gather, rope):
+    """Two sequences of four tiles a CTA with three stages: the tiles after the first stalled
+    ones belong partly to the next sequence.  A consumer that took a stage which never filled
+    would append the earlier tile's new row there, at the earlier sequence's slot."""
+    dev, d, k, W = cuda_device, 128, 64, 192
+    rows = 256 if gather else k
+
+    def dims_of(B):
+        return cmc.CmcDims(B, 1, 4, 1, d, rows, k, W)
+
+    B = 2 * cmc.decode_attn_plan(dims_of(1 << 14), rope=rope)[0]
+    dims = dims_of(B)
+    assert cmc.decode_attn_plan(dims, rope=rope) == (B // 2, 1)
+    g = torch.Generator(device=dev).manual_seed(3)
+
+    def rand(*shape):
+        return torch.randn(shape, generator=g, device=dev).to(torch.bfloat16)
+
+    t1 = [rand(B, 1, 1, rows, d) for _ in range(2)]
+    ring = [rand(B, 1, 1, W, d) for _ in range(2)]
+    new = [rand(B, 1, 1, d) for _ in range(2)]
+    q = rand(B, 1, 4, d)
+    idx = (torch.rand((B, rows), generator=g, device=dev).topk(k, dim=1).indices.to(torch.int32)
+           if gather else None)
+    pos = W + (37 * torch.arange(B, device=dev)) % W
+    before, slot = [t.clone() for t in ring], pos % W
+    ws = cmc.DecodeWorkspace(dims, dev)
+    torch.cuda.synchronize(dev)
+    assert cmc.lib().cmc_test_stall_attention_waits(1) == 0
+    try:
+        kw = dict(rope_theta=ROPE_THETA, rope_offset=k) if rope else {}
+        cmc.decode_step(q, *t1, idx, *ring, pos, *new, workspace=ws, **kw)
+        flags = ws.status()
+    finally:
+        assert cmc.lib().cmc_test_stall_attention_waits(0) == 0
+    assert flags & DEVFLAG_TIMEOUT
+    own = torch.arange(W, device=dev)[None, :] == slot[:, None]
+    for got, want in zip(ring, before):
+        changed = (got != want).any(dim=-1)[:, 0, 0]
+        assert not (changed & ~own).any(), f"{int((changed & ~own).sum())} rows of other tokens changed"
