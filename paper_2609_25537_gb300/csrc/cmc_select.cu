@@ -127,9 +127,24 @@ cosine_scores_kernel(const float* __restrict__ qv, const float* __restrict__ ban
 // Calls back to back, a CTA per row -> a warp per row: 2 x 8,192 CMEs of 768
 // features 31 -> 16 us, 24 x 826 of 1,280 39 -> 26, 16 x 2,000 of 2,048 66 -> 45.  At
 // 4,096 features a CTA per row streams at 6.5 TB/s, and stays.
+//
+// A lane's dot product and squared norm go through four accumulators each, one
+// per float4 component, joined before the butterfly: D / 128 additions one after
+// the other.  With one each (D / 32) the scores were further from 64 bits than the
+// CTA per row's (D / 256): at 2,048 features 1.66e-7 of their norm against 1.17e-7,
+// now 1.17e-7.  The question's norm, the same for a whole bank, stays with one:
+// four more registers cost loads in flight (16 x 20,000 of 512: 152 us before, 157
+// now, 182 with four there too).
 constexpr int kWarpScoreD = 2048;
 constexpr int kWarpScoreCtas = 3;   // per SM
 constexpr int kWarpScoreLoads = 8;  // float4s a lane has in flight
+
+__device__ __forceinline__ void fma_f4(float4& acc, const float4& a, const float4& b) {
+  acc.x = fmaf(a.x, b.x, acc.x);
+  acc.y = fmaf(a.y, b.y, acc.y);
+  acc.z = fmaf(a.z, b.z, acc.z);
+  acc.w = fmaf(a.w, b.w, acc.w);
+}
 
 __global__ void __launch_bounds__(kScoreThreads, kWarpScoreCtas)
 cosine_scores_warp_kernel(const float* __restrict__ qv, const float* __restrict__ bank, int N, int D,
@@ -148,7 +163,9 @@ cosine_scores_warp_kernel(const float* __restrict__ qv, const float* __restrict_
                             : r / N;
     const float4* m = reinterpret_cast<const float4*>(bank + r * D);
     const float4* q = reinterpret_cast<const float4*>(qv + b * D);
-    float dot = 0.f, mm = 0.f, qq = 0.f;
+    float4 dot4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 mm4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    float qq = 0.f;
     for (int i0 = lane; i0 < D4; i0 += 32 * U) {
       float4 a[U], c[U];
 #pragma unroll
@@ -159,14 +176,16 @@ cosine_scores_warp_kernel(const float* __restrict__ qv, const float* __restrict_
         c[u] = i0 + 32 * u < D4 ? __ldg(q + i0 + 32 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        dot = fmaf(a[u].x, c[u].x, dot); dot = fmaf(a[u].y, c[u].y, dot);
-        dot = fmaf(a[u].z, c[u].z, dot); dot = fmaf(a[u].w, c[u].w, dot);
-        mm = fmaf(a[u].x, a[u].x, mm); mm = fmaf(a[u].y, a[u].y, mm);
-        mm = fmaf(a[u].z, a[u].z, mm); mm = fmaf(a[u].w, a[u].w, mm);
-        qq = fmaf(c[u].x, c[u].x, qq); qq = fmaf(c[u].y, c[u].y, qq);
-        qq = fmaf(c[u].z, c[u].z, qq); qq = fmaf(c[u].w, c[u].w, qq);
+        fma_f4(dot4, a[u], c[u]);
+        fma_f4(mm4, a[u], a[u]);
+        qq = fmaf(c[u].x, c[u].x, qq);
+        qq = fmaf(c[u].y, c[u].y, qq);
+        qq = fmaf(c[u].z, c[u].z, qq);
+        qq = fmaf(c[u].w, c[u].w, qq);
       }
     }
+    float dot = (dot4.x + dot4.y) + (dot4.z + dot4.w);
+    float mm = (mm4.x + mm4.y) + (mm4.z + mm4.w);
 #pragma unroll
     for (int off = 16; off >= 1; off >>= 1) {
       dot += __shfl_xor_sync(0xffffffffu, dot, off);
