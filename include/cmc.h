@@ -190,7 +190,8 @@ CMC_API size_t cmc_score_select_workspace_size(int B, int N);
  * counter in the workspace tells it) selects that sequence's top k, starting
  * from the histogram the scoring CTAs built.  Larger
  * banks, or no workspace, take two launches (scoring, then selection; the
- * histogram serves the second up to 32,768 CMEs).  All give the same selection.
+ * histogram serves the second up to 32,768 CMEs, or 16,384 if N is no multiple
+ * of 4 or scores_out not 16-byte aligned).  All give the same selection.
  *
  * Scores are computed in fp32 with a fixed summation order, so equal rows get
  * bit-identical scores.  Equal scores go to the lower index; -0 equals +0.  A

@@ -823,10 +823,26 @@ __device__ __forceinline__ void fused_select_impl(const FusedArgs& a, int b) {
   const float* sc = a.scores + static_cast<long long>(b) * N;
   uint32_t* ghist = a.hist + static_cast<long long>(b) * kHistTop;
   uint32_t key[KPT];
+  if (KPT >= 4 && (N & 3) == 0 && (reinterpret_cast<uintptr_t>(a.scores) & 15) == 0) {
+    // four at a time: a thread's keys are consecutive, so a warp's load of one
+    // word each touches 32 sectors, KPT times over (see topk_hist_kernel)
 #pragma unroll
-  for (int e = 0; e < KPT; ++e) {
-    const int j = tid * KPT + e;
-    key[e] = (topk && j < N) ? orderable(__ldcg(sc + j)) : 0u;
+    for (int e = 0; e + 3 < KPT; e += 4) {
+      const int j = tid * KPT + e;
+      const float4 v = (topk && j < N) ? __ldcg(reinterpret_cast<const float4*>(sc + j))
+                                       : make_float4(0.f, 0.f, 0.f, 0.f);
+      const bool in = topk && j < N;
+      key[e] = in ? orderable(v.x) : 0u;
+      key[e + 1] = in ? orderable(v.y) : 0u;
+      key[e + 2] = in ? orderable(v.z) : 0u;
+      key[e + 3] = in ? orderable(v.w) : 0u;
+    }
+  } else {
+#pragma unroll
+    for (int e = 0; e < KPT; ++e) {
+      const int j = tid * KPT + e;
+      key[e] = (topk && j < N) ? orderable(__ldcg(sc + j)) : 0u;
+    }
   }
   // this thread's two bins of the top-bits histogram, in flight with the keys
   uint32_t ga = 0u, gb = 0u;
@@ -1032,8 +1048,13 @@ score_select_fused_kernel(const __grid_constant__ FusedArgs a) {
 // topk_select_cluster_kernel) -> with this one, the CTA-per-row scoring before
 // either: 4 x 1,024 CMEs 21.1 -> 18.0 us, 32 x 2,048 178 -> 165, 1 x 8,192 of 4,096
 // features 46 -> 30, 1 x 4,000 of 1,280 20.3 -> 11.5.  Without a workspace, for k
-// outside 1 .. N - 1 and above kHistMaxN CMEs the others run.
+// outside 1 .. N - 1 and above kHistMaxN CMEs the others run.  So does the cluster
+// kernel for more than kHistWordN CMEs whose scores cannot be read four at a time (N no
+// multiple of 4, or scores_out not 16-byte aligned).  1 x N of 4,096 features, the
+// cluster kernel / four keys at a time / one: N = 16,384 59.7 / 52.2 / 55.2 us, 20,480
+// 71.2 / 66.2 / 74.1, 32,768 101.0 / 97.1 / 109.3.
 constexpr int kHistMaxN = 32 * kFusedThreads;
+constexpr int kHistWordN = 16 * kFusedThreads;
 
 template <int KPT>
 __global__ void __launch_bounds__(kFusedThreads)
@@ -1118,7 +1139,8 @@ static int launch_score_select(const float* question_emb, const float* cme_bank,
   const long long cap = static_cast<long long>(sm_count()) * (by_warp ? kWarpScoreCtas : 2048 / kScoreThreads);
   if (blocks > cap) blocks = cap;
   // the histograms follow the counters in the workspace
-  const bool use_hist = counters && N <= kHistMaxN && k > 0 && k < N;
+  const bool by_four = (N & 3) == 0 && aligned16(sc);
+  const bool use_hist = counters && N <= (by_four ? kHistMaxN : kHistWordN) && k > 0 && k < N;
   unsigned int* hist = nullptr;
   if (use_hist)
     hist = reinterpret_cast<unsigned int*>(reinterpret_cast<char*>(counters) +

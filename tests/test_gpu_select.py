@@ -304,3 +304,28 @@ def test_scores_of_warp_rows_are_as_exact_as_a_cta_s(cuda_device, D):
     ref = torch.nn.functional.cosine_similarity(bank.double(), q.double()[:, None], dim=2, eps=0.0)
     err = ((scores.double() - ref).norm() / ref.norm()).item()
     assert err <= 1.35e-7, f"{err:.3e}"
+
+
+@pytest.mark.parametrize("N,offset", [(2052, 0), (2052, 1), (4100, 0), (4102, 0), (8196, 0),
+                                      (16380, 0), (16383, 0), (16384, 2), (16388, 0), (16388, 1),
+                                      (16390, 0), (32764, 0), (32767, 0), (32768, 3)])
+def test_select_reads_scores_by_four_or_one(cuda_device, N, offset):
+    """Scores at 16-byte boundaries (N a multiple of 4) or not, on both sides of the sizes where
+    the selection's kernel changes; the last keys belong to a thread that has a part of its own
+    only.  Ties as above, against a sort."""
+    B, D = 2, 36
+    rng = np.random.default_rng(N + offset)
+    q = rng.integers(-40, 41, size=(B, D)).astype(np.float32)
+    q[:, 0] = 41.0
+    ws = torch.zeros(cmc.score_select_workspace_size(B, N), dtype=torch.uint8, device=cuda_device)
+    scores = torch.empty(B * N + offset, device=cuda_device)[offset:].view(B, N)
+    axis = rng.integers(0, D, size=(B, N))
+    bank = np.zeros((B, N, D), dtype=np.float32)
+    bank[np.arange(B)[:, None], np.arange(N)[None, :], axis] = 1.0
+    for k in (1, N // 3, N - 1):
+        got = cmc.score_select(dev_f32(q, cuda_device), dev_f32(bank, cuda_device), k,
+                               scores_out=scores, workspace=ws).cpu().numpy()
+        for b in range(B):
+            order = np.lexsort((np.arange(N), -q[b, axis[b]]))
+            np.testing.assert_array_equal(got[b], np.sort(order[:k]), err_msg=f"k={k} b={b}")
+    assert not ws[-(-B * N * 4 // 256) * 256:].any()
