@@ -61,10 +61,37 @@ def test_bridge_epilogue_many_rows(cuda_device):
 
 
 @pytest.mark.parametrize("D,per_sm", [(4, 8), (2048, 8), (2052, 4), (4096, 4), (4100, 2), (8192, 2),
-                                      (8196, 1), (16384, 1)])
+                                      (8196, 2), (10244, 2), (12288, 2), (14336, 2), (16384, 2)])
 @pytest.mark.parametrize("affine", [False, True])
 def test_bridge_epilogue_thread_counts(cuda_device, D, per_sm, affine):
     """The row lengths where a CTA's threads change, over three more rows than the most CTAs
     that are resident, so that some walk two (gamma and beta kept from the first)."""
     sms = torch.cuda.get_device_properties(cuda_device).multi_processor_count
     _case(per_sm * sms + 3, D, 0.8, 2.0, affine, cuda_device, in_place=True)
+
+
+@pytest.mark.parametrize("D,per_sm", [(1540, 101), (1664, 101), (2052, 21), (2304, 31), (3328, 38),
+                                      (3072, 61), (4076, 60), (1924, 81), (2048, 81), (2820, 51),
+                                      (4096, 51)])
+@pytest.mark.parametrize("gain,shift", [(False, False), (True, True), (True, False), (False, True)])
+def test_bridge_epilogue_many_rows_as_few(cuda_device, D, per_sm, gain, shift):
+    """So many rows that the variant for many rows takes them (with or without gamma and beta, as
+    the width has it): the same bits as from calls of a few rows each where those take 128 threads
+    too.  With gamma or beta and over 2,048 features they take 256, and add in another order: the
+    three sums are off by some ten roundings of 2^-24 each, 2e-6 in all."""
+    sms = torch.cuda.get_device_properties(cuda_device).multi_processor_count
+    rows = per_sm * sms + 5
+    g = torch.Generator(device=cuda_device).manual_seed(D)
+    x = torch.randn(rows, D, device=cuda_device, generator=g) * 2.0 + 0.3
+    kw = {}
+    if gain:
+        kw["gamma"] = torch.randn(D, device=cuda_device, generator=g) * 0.02
+    if shift:
+        kw["beta"] = torch.randn(D, device=cuda_device, generator=g) * 0.005
+    few = torch.cat([cmc.bridge_epilogue(part, 0.8, **kw) for part in x.split(10 * sms)])
+    many = cmc.bridge_epilogue(x, 0.8, **kw)
+    if kw and D > 2048:
+        assert ((many - few).norm(dim=1) <= 2e-6 * few.norm(dim=1)).all()
+    else:
+        assert torch.equal(many, few)
+    assert torch.equal(cmc.bridge_epilogue(x, 0.8, out=x, **kw), many)
