@@ -329,6 +329,7 @@ __device__ __forceinline__ void locate_window(const LocateArgs& la, int b, int N
   if (tid == 0) {
     for (int w = 1; w < static_cast<int>(blockDim.x >> 5); ++w)
       if (wbest[w] > best || (wbest[w] == best && wbidx[w] < bi)) { best = wbest[w]; bi = wbidx[w]; }
+    if (bi >= N) bi = 0;  // every norm is NaN: no row was above -1
     const long long alpha = la.chunk_offset[static_cast<long long>(b) * N + bi];
     long long st = static_cast<long long>(la.ctx_len[b]) - la.W;
     const long long centred = alpha - la.W / 2;

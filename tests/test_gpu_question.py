@@ -129,3 +129,17 @@ def test_kept_workspaces_of_two_shapes_of_one_size(cuda_device, first, second):
             _norm_gap_ok(bank)
             offs = np.tile(np.arange(N, dtype=np.int32) * 4, (B, 1))
             _check(tokens, None, bank, N // 8, offs, np.full(B, 4 * N, dtype=np.int32), 64, cuda_device)
+
+
+@pytest.mark.parametrize("B,N", [(1, 64), (2, 3000), (1, 40000)])
+def test_a_bank_without_a_norm_locates_its_first_chunk(cuda_device, B, N):
+    """CMEs that are all NaN (one launch, the histogram search, the cluster kernel): no norm is the
+    largest, and the localisation reads no chunk offset past the bank's.  The selection of such a
+    bank is not specified; it stays within the bank."""
+    tokens = torch.ones(B, 3, 64, device=cuda_device)
+    bank = torch.full((B, N, 64), float("nan"), device=cuda_device)
+    offs = 7 + torch.arange(N, dtype=torch.int32, device=cuda_device).repeat(B, 1)
+    clen = torch.full((B,), N, dtype=torch.int32, device=cuda_device)
+    _, idx, alpha, start = cmc.question_select(tokens, bank, N // 4, chunk_offset=offs, ctx_len=clen, W=8)
+    assert alpha.cpu().tolist() == [7] * B and start.cpu().tolist() == [3] * B
+    assert 0 <= int(idx.min()) and int(idx.max()) < N
