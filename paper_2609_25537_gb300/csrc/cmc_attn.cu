@@ -831,8 +831,16 @@ __device__ __forceinline__ void seq_run_done(const AttnParams& p, int b, int til
 // the CTA's tiles through NST shared-memory stages; stage s is handed over by
 // full[s] (its bytes have landed and its header is written) and handed back
 // by empty[s] (every consumer warp is done with it).
+//
+// 144 registers a thread at d = 128: two CTAs put three warps on some of an SM's
+// four schedulers, and those leave room for two warps of 40 registers of another
+// kernel.  At up to 168 nothing fitted beside a full grid, and the staging copies
+// and combine launches of other streams waited for it: two streams of 448 units
+// (split, with staging copies) 130 us a pass, now 105, four of them 205 and 175,
+// 320 units on one stream 175.5 and 171.2.  At 128 8 x (30 + 130) keys take 1.5 % more,
+// at 144 the same as at 168 (150.4 us), 32 layers of 128 + 512 keys 228.2 and 227.6.
 template <int D, int G, bool FUSED, int NST, bool ROPE>
-__global__ void __launch_bounds__(kThreads + 32, D == 64 ? 4 : 2)
+__global__ void __maxnreg__(D == 64 ? 96 : 144)
 two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) {
   using S = Stage<D, G, ROPE>;
   constexpr int KS = D / 16;  // k-steps of the Q K^T product
