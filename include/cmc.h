@@ -410,12 +410,12 @@ CMC_API int cmc_read_status(void* workspace, int clear, uint32_t* flags, void* s
 /* Tuning of the attention launches (cmc_two_tier_decode_attn,
  * cmc_decode_step, cmc_decode_step_rope) made afterwards, from any thread:
  * before its grid dependency wait every CTA asks L2 to prefetch the K/V boxes
- * of at most its first `tiles` tiles (64 keys each; a launch takes fewer where
- * its plan gains from that: two when a cluster of CTAs shares a unit, four, or
- * at d = 64 two, when CTAs take whole units), so that under programmatic
+ * of its first `tiles` tiles (64 keys each), so that under programmatic
  * dependent launch they stream in while the kernel before it on the stream
  * drains.  A hint only: results do not depend on it.  Default 5, for one stream
- * of launches; 0 was best when
+ * of launches; with the default a launch takes fewer where its plan gains from
+ * that (two when a cluster of CTAs shares a unit, four, or at d = 64 two, when
+ * CTAs take whole units), any other depth is taken as it is.  0 was best when
  * four independent requests' launches ran on four streams (their launches
  * already overlap).  CMC_ERR_RANGE unless 0 <= tiles <= 64. */
 CMC_API int cmc_set_l2_prefetch_tiles(int tiles);

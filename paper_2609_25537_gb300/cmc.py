@@ -428,8 +428,9 @@ def decode_step(q, tier1_k, tier1_v, idx, ring_k, ring_v, pos, k_new, v_new, *,
 
 def set_l2_prefetch_tiles(tiles: int) -> None:
     """Box tiles per CTA the attention launches made afterwards prefetch into
-    L2 before their grid dependency wait, at most (a hint); see
-    cmc_set_l2_prefetch_tiles.  Default 5 (one stream of launches); 0 suits
+    L2 before their grid dependency wait (a hint); see
+    cmc_set_l2_prefetch_tiles.  Default 5 (one stream of launches; fewer where
+    a launch's plan gains from that); 0 suits
     several streams of independent requests' launches."""
     check(lib().cmc_set_l2_prefetch_tiles(int(tiles)), "cmc_set_l2_prefetch_tiles")
 

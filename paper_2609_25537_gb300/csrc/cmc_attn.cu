@@ -1782,7 +1782,7 @@ static int plan_attn(long long total_tiles, int tpu, AttnPlan* pl) {
   return CMC_OK;
 }
 
-// The most tiles a CTA of a plan gains from prefetching (of the setting's).  us a
+// The most tiles a CTA of a plan gains from prefetching (of the default).  us a
 // round at depth 1 / 2 / 3 / 5, two requests in turn on one stream:
 //   clusters:     16 x (64 + 512 keys) 67.5 / 68.2 / 69.3 / 71.4, the same as
 //                 separate append and attention 42.0 / 43.8 / 47.1 / 50.1, 12 x
@@ -1837,7 +1837,9 @@ static int launch_attn(const AttnMaps& maps, const AttnParams& p0, long long tot
   p.base = static_cast<int>(pl.base);
   p.rem = static_cast<int>(pl.rem);
   p.cm = pl.cm;
-  p.l2_prefetch = p0.l2_prefetch < prefetch_cap(pl, D) ? p0.l2_prefetch : prefetch_cap(pl, D);
+  // the default, but not a depth that the caller has set, is capped by the plan
+  if (p0.l2_prefetch == kL2PrefetchTiles && prefetch_cap(pl, D) < kL2PrefetchTiles)
+    p.l2_prefetch = prefetch_cap(pl, D);
   p.slice = pl.cm > 0 ? (G * D / 4 + pl.cm - 1) / pl.cm : 0;
   if (p.idx) {
     // Gathered Tier-1: each CTA begins with a pipeline's depth of ring tiles,
