@@ -845,7 +845,7 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
   using S = Stage<D, G, ROPE>;
   constexpr int KS = D / 16;  // k-steps of the Q K^T product
   constexpr int DP = merge_row_floats(D);  // padded row of the merge buffer
-  extern __shared__ uint8_t smem_raw[];
+  extern __shared__ __align__(16) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* aux0 = smem + NST * S::kBytes;                              // NST aux areas
   uint8_t* meta0 = aux0 + NST * S::kAuxBytes;                          // kMetaSlots slots
