@@ -676,7 +676,7 @@ struct FusedArgs {
   int32_t* idx_out;       // [B, k]
   LocateArgs la;          // la.sqnorm: also write squared norms and localise
   unsigned int* hist;     // [B, kHistTop]: counts of the scores' top 11 key bits (zero before,
-                          // zero after; left alone for k = 0 and k = N)
+                          // zero after); NULL for k = 0 and k = N, which search nothing
 };
 
 // Exclusive prefix sum over the block of one value per thread (warps in
@@ -828,7 +828,7 @@ __device__ __forceinline__ void fused_select_impl(const FusedArgs& a, int b) {
   const int N = a.N, k = a.k;
   const bool topk = k > 0 && k < N;
   const float* sc = a.scores + static_cast<long long>(b) * N;
-  uint32_t* ghist = a.hist + static_cast<long long>(b) * kHistTop;
+  uint32_t* ghist = a.hist + static_cast<long long>(b) * kHistTop;  // used for a search only
   uint32_t key[KPT];
   if (KPT >= 4 && (N & 3) == 0 && (reinterpret_cast<uintptr_t>(a.scores) & 15) == 0) {
     // four at a time: a thread's keys are consecutive, so a warp's load of one
@@ -1007,8 +1007,7 @@ score_select_fused_kernel(const __grid_constant__ FusedArgs a) {
       if (sm > 0.f && qq > 0.f) sc = sd / (sqrtf(sm) * sqrtf(qq));
       if (sc == 0.f) sc = 0.f;  // -0 -> +0, so that -0 and +0 tie
       a.scores[r0 + warp] = sc;
-      // only for a search, which puts the counts back to zero
-      if (a.k > 0 && a.k < a.N)
+      if (a.hist)  // only for a search, which puts the counts back to zero
         atomicAdd(a.hist + static_cast<long long>(b) * kHistTop + (orderable(sc) >> 21), 1u);
       if (a.la.sqnorm) a.la.sqnorm[r0 + warp] = sm;
       rsq_s[warp] = sm;
@@ -1117,9 +1116,13 @@ static int launch_score_select_fused(const float* question_emb, const float* cme
   a.counters = counters;
   a.idx_out = idx_out;
   a.la = la;
-  // the histograms follow the counters in the workspace
-  a.hist = reinterpret_cast<unsigned int*>(reinterpret_cast<char*>(counters) +
-                                           align_up(static_cast<size_t>(B) * sizeof(unsigned int), 256));
+  // the histograms follow the counters in the workspace (a NULL here, instead of k
+  // compared with N in the kernel, keeps its registers: four requests of 1,024 x
+  // 4,096 with their compaction 75.6 us, and 79.9)
+  a.hist = nullptr;
+  if (k > 0 && k < N)
+    a.hist = reinterpret_cast<unsigned int*>(reinterpret_cast<char*>(counters) +
+                                             align_up(static_cast<size_t>(B) * sizeof(unsigned int), 256));
   const long long ctas = static_cast<long long>(B) * N / R;
   return launch_pdl(score_select_fused_kernel, dim3(static_cast<unsigned>(ctas)),
                     dim3(kFusedThreads), fused_smem_bytes(), s, a);
