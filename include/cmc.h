@@ -119,9 +119,9 @@ CMC_API size_t cmc_denoise_workspace_size(int B, int n_max);
  *               on completion its first B * n_max bytes hold each token's
  *               threshold-test result (1 passed, 0 not or past n_tokens)
  *
- * When the contexts' 32-token tiles fit one CTA per SM (B * ceil(n_max / 32)
- * <= SM count), the whole call is one kernel launch: the CTA that finishes a
- * context's last tile also walks its keep-minimum and writes kept_idx.
+ * For n_max of up to 8,192 (256 tiles of 32 tokens a context) the whole call
+ * is one kernel launch: the CTA that finishes a context's last tile also walks
+ * its keep-minimum and writes kept_idx.
  *
  * Limits: 1 <= B <= 65535, 1 <= n_max <= 2^24, 4 <= H <= 65536, H % 4 == 0,
  * 1 <= g <= 8, keep_every >= 0, tau finite.

@@ -327,7 +327,7 @@ __device__ __forceinline__ void consumer_sync() {
 }
 
 // --- thread-block cluster: barrier (every thread of every CTA of the
-// cluster arrives, then waits) and loads from a peer CTA's shared memory.
+// cluster arrives, then waits) and stores into a peer CTA's shared memory.
 __device__ __forceinline__ void cluster_arrive() {
   asm volatile("barrier.cluster.arrive.release;\n" ::: "memory");
 }

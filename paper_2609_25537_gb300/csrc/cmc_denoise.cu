@@ -187,8 +187,8 @@ denoise_pass_kernel(const float* __restrict__ emb, const int32_t* __restrict__ n
   const int r0 = warp * TPW;  // this warp's first token row in the tile
   // The context and the first token of a tile: a CTA's first before the grid
   // dependency wait, in 32 bits where the tile numbers fit.  With the -1s
-  // written after the first chunks are requested, 1 to 2 % of a call (4 contexts of
-  // 4,096 tokens 22.5 -> 22.0 us, 8 of 8,000 50.8 -> 50.0).
+  // written after the first chunks are requested, about 1 % of a call (four calls
+  // of 4,096 tokens 39.1 -> 38.6 us, one of 65,536 64.0 -> 63.4).
   int b, i0;
   auto place = [&](long long t) {
     if (tiles <= 0x7fffffffll)

@@ -10,14 +10,15 @@
 //
 // Larger banks, two launches:
 //  1. cosine_scores_kernel -- one CTA of 256 threads per CME row (grid-stride
-//     over rows), or cosine_scores_warp_kernel, one warp per row, for rows of
-//     up to 2,048 features: every thread streams its share of the row with 16-byte loads
+//     over rows): every thread streams its share of the row with 16-byte loads
 //     issued four at a time, accumulating m.q, m.m and q.q in fp32; the
 //     partial sums meet in a fixed tree (warp shuffles, then the eight warps
-//     in order), so equal rows produce bit-identical scores.  HBM-bound:
-//     4*D bytes per row, with a whole row per CTA in flight.
+//     in order).  Rows of up to 2,048 features: cosine_scores_warp_kernel, one
+//     warp per row, a lane's loads issued eight at a time, its sums joined by
+//     the shuffles alone.  Equal rows produce bit-identical scores in either.
+//     HBM-bound: 4*D bytes per row.
 //  2. topk_hist_kernel -- one CTA per sequence of up to 32,768 CMEs, when the
-//     call has a workspace for the histogram that the scoring builds (see
+//     call has a workspace for the histogram that the scoring builds (limits
 //     there); otherwise topk_select_kernel, one CTA per sequence (above 8,192
 //     CMEs topk_select_cluster_kernel: a cluster of 8).  Scores are mapped to
 //     order-preserving uint32 keys; a 4-pass MSB radix select (8 bits a pass)

@@ -773,9 +773,9 @@ PARTIAL = [(1, 1), (15, 17), (16, 48), (30, 130), (48, 49), (63, 65), (65, 127),
 @pytest.mark.parametrize("k,W", PARTIAL)
 @pytest.mark.parametrize("plan", ["cluster", "whole units"])
 def test_partial_tiles_and_partly_filled_rings(cuda_device, plan, k, W, mode):
-    """Sizes around the 16-row boxes of a partial tile and the 64-row tiles, with rings from empty
-    to wrapped, so that ring tiles without a key are left out in the middle of a launch: one
-    unit shared by a cluster, and several units and sequences in one CTA."""
+    """Sizes around a warp's 16 keys of a tile and the 64-key tiles, with rings from empty to
+    wrapped, so that a launch has ring tiles without a key between others: one unit shared by a
+    cluster, and several units and sequences in one CTA."""
     fills = sorted({0, 1, 15, 16, 17, W // 3, W // 2, W - 1, W, 63, 64, 65} & set(range(W + 1)))
     B, L = (len(fills), 1) if plan == "cluster" else (4 * len(fills), 16)
     w = WORKLOADS["tiny"].with_(name="partial", B=B, L=L, N=128, k=k, W=W, T=3,

@@ -3,10 +3,11 @@
 The selected index set is compared bit-exactly (as an ordered array); scores
 within 1e-5 absolute (fp32 accumulation over D <= 4096 terms of a cosine).
 
-Both launch paths run on every case: one launch (a workspace given, N <= 8192,
-D <= 4096: the CTA that completes a sequence's scores selects it) and two
-launches (no workspace, scores_out given, reached through the C ABI; also the
-path of larger banks).  They must select the same rows."""
+Both launch paths run on every case: with a workspace (the binding's) one launch
+for small banks (N <= 2048, D <= 4096, one wave of CTAs: the CTA that completes a
+sequence's scores selects it), the histogram search after the scoring launch for
+larger ones; and two launches without a workspace (scores_out given, reached
+through the C ABI).  They must select the same rows."""
 
 import ctypes
 
