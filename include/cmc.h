@@ -425,8 +425,10 @@ CMC_API int cmc_set_l2_prefetch_tiles(int tiles);
  * attention launches made afterwards (cmc_two_tier_decode_attn,
  * cmc_decode_step, cmc_decode_step_rope, from any thread) expects 16 bytes
  * more than its loads deliver, so no stage ever completes: each CTA's first
- * wait gives up after its 1 s limit, the CTA's other waits end at once, the
- * launch returns and the workspace's status word gets CMC_DEVFLAG_TIMEOUT.
+ * wait gives up after its 1 s limit, the CTA's other waits end at once (but for a
+ * cluster's wait for what its CTAs store into each other, which is stalled
+ * likewise and gives up after 3 s), the launch returns and the workspace's status
+ * word gets CMC_DEVFLAG_TIMEOUT.
  * Outputs, ring and pos of such a call are invalid, and its workspace must be
  * zero-filled again.  on == 0 restores normal operation.  Always CMC_OK. */
 CMC_API int cmc_test_stall_attention_waits(int on);

@@ -369,12 +369,23 @@ __device__ __forceinline__ void st_peer_f2(uint32_t addr, float x, float y, uint
       "f"(x), "f"(y), "r"(bar)
       : "memory");
 }
+// Out of line: the wait it belongs to is on every cluster's way to its output
+// (inlined, clusters of 8 took 1 % more).
+__device__ __noinline__ void peers_gave_up() {
+  *static_cast<volatile int*>(&attn_abort) = 1;
+  cluster_sync_all();  // over the threads of the cluster that have not ended
+  const uint32_t t0 = global_ns32();
+  for (uint32_t it = 0; it < (1u << 16) && global_ns32() - t0 < kDrainNs; ++it) __nanosleep(1000);
+}
+
 // Waits for the peers' stores counted by `bar` (phase 0).  Unlike the pipeline's
 // waits it does not end with the CTA's abort flag: a CTA must not leave while
 // its peers still store into its shared memory.  Peers that gave up have done
 // so within kWaitNs of the cluster's start and store all the same, so the
-// limit (kPeerWaitNs) lies well behind theirs.
-__device__ __forceinline__ bool mbar_wait_peers(uint64_t* bar) {
+// limit (kPeerWaitNs) lies well behind theirs.  Should it pass even so, the CTA
+// stays until every peer has come to the same point or has ended (each does:
+// its own waits are bounded), and kDrainNs longer for stores on the way.
+__device__ __forceinline__ void mbar_wait_peers(uint64_t* bar) {
   const uint32_t t0 = global_ns32();
   for (uint32_t it = 0; it < kMaxWaitPolls; ++it) {
     uint32_t ok;
@@ -384,11 +395,10 @@ __device__ __forceinline__ bool mbar_wait_peers(uint64_t* bar) {
         : "=r"(ok)
         : "r"(smem_addr(bar))
         : "memory");
-    if (ok) return true;
+    if (ok) return;
     if (global_ns32() - t0 > kPeerWaitNs) break;
   }
-  *static_cast<volatile int*>(&attn_abort) = 1;
-  return false;
+  peers_gave_up();
 }
 
 // ---------------------------------------------------------------------------
@@ -898,7 +908,7 @@ two_tier_attn_kernel(const __grid_constant__ AttnMaps maps, const AttnParams p) 
     const int mine = min(max(G * D / 4 - j_begin * p.slice, 0), p.slice);
     mbar_init(&recv_bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    mbar_arrive_expect_tx(&recv_bar, static_cast<uint32_t>(p.cm * (mine * 16 + G * 8)));
+    mbar_arrive_expect_tx(&recv_bar, static_cast<uint32_t>(p.cm * (mine * 16 + G * 8)) + p.stall_tx);
   }
   __syncthreads();
   // The cluster's only barrier: the receive barriers exist before a peer's

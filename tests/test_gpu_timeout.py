@@ -5,7 +5,9 @@ more than its loads deliver, so that no stage's barrier phase ever completes
 (a wait that nothing ends: no access leaves its buffer and nothing traps).
 Each CTA's first wait then gives up after its 1 s limit, the CTA's other
 waits end at once, the producer warp gives its issued loads 2 ms to land, and
-the call reports CMC_DEVFLAG_TIMEOUT in the workspace's status word.
+the call reports CMC_DEVFLAG_TIMEOUT in the workspace's status word.  In a
+cluster plan the wait for the peers' stores is stalled too: it gives up after 3 s,
+meets the peers at a cluster barrier and gives their stores 2 ms.
 
 Checked: the call returns, the flag is raised, and the context stays usable
 -- with the hook off and the ring, pos and workspace restored, the same step
@@ -130,3 +132,33 @@ def test_stalled_call_leaves_other_ring_rows_alone(cuda_device, gather, rope):
     for got, want in zip(ring, before):
         changed = (got != want).any(dim=-1)[:, 0, 0]
         assert not (changed & ~own).any(), f"{int((changed & ~own).sum())} rows of other tokens changed"
+
+
+@pytest.mark.parametrize("B,k,W", [(19, 64, 64), (12, 128, 192), (1, 640, 640)])
+def test_stalled_clusters_end(cuda_device, B, k, W):
+    """Clusters of 2, 3 and 8 CTAs (some of their CTAs with fewer tiles than others) whose waits
+    for each other run out: the call ends, flagged, and the next one on the device is right."""
+    dev, d = cuda_device, 128
+    g = torch.Generator(device=dev).manual_seed(B)
+
+    def rand(*shape):
+        return torch.randn(shape, generator=g, device=dev).to(torch.bfloat16)
+
+    t1 = [rand(B, 1, 8, k, d) for _ in range(2)]
+    ring = [rand(B, 1, 8, W, d) for _ in range(2)]
+    q, pos = rand(B, 1, 32, d), torch.full((B,), W, dtype=torch.int64, device=dev)
+    args = (q, *t1, None, *ring, pos)
+    want = cmc.two_tier_decode_attn(*args)
+    ws = cmc.DecodeWorkspace(cmc.dims_of(q, t1[0], None, ring[0]), dev)
+    torch.cuda.synchronize(dev)
+    assert cmc.lib().cmc_test_stall_attention_waits(1) == 0
+    try:
+        t0 = time.perf_counter()
+        cmc.two_tier_decode_attn(*args, workspace=ws)
+        flags = ws.status()
+        elapsed = time.perf_counter() - t0
+    finally:
+        assert cmc.lib().cmc_test_stall_attention_waits(0) == 0
+    assert flags & DEVFLAG_TIMEOUT
+    assert 2.9 <= elapsed < 30.0
+    assert torch.equal(cmc.two_tier_decode_attn(*args), want)
