@@ -417,7 +417,8 @@ CMC_API int cmc_read_status(void* workspace, int clear, uint32_t* flags, void* s
  * that (two when a cluster of CTAs shares a unit, four, or at d = 64 two, when
  * CTAs take whole units), any other depth is taken as it is.  0 was best when
  * four independent requests' launches ran on four streams (their launches
- * already overlap).  CMC_ERR_RANGE unless 0 <= tiles <= 64. */
+ * already overlap); with 0, staging copies of 32 KB or more (cmc_stage_copies) also
+ * let the launch after them start with their end only.  CMC_ERR_RANGE unless 0 <= tiles <= 64. */
 CMC_API int cmc_set_l2_prefetch_tiles(int tiles);
 
 /* Test hook for the failure path of the attention kernels (not part of the

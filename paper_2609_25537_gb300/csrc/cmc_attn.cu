@@ -1708,6 +1708,7 @@ constexpr int kStages = 3;
 constexpr int kL2PrefetchTiles = 5;
 constexpr int kMaxL2PrefetchTiles = 64;
 static std::atomic<int> g_l2_prefetch_tiles{kL2PrefetchTiles};
+int l2_prefetch_setting() { return g_l2_prefetch_tiles.load(std::memory_order_relaxed); }
 
 // Launch plan of one attention call on the current device.
 struct AttnPlan {
@@ -2055,7 +2056,7 @@ static int run_attention(const void* q, const void* tier1_k, const void* tier1_v
   const float sc = scale > 0.f ? scale : 1.0f / sqrtf(static_cast<float>(m.d));
   p.scale_log2 = sc * 1.4426950408889634f;
   p.rope_offset = rope ? rope_offset : 0;
-  p.l2_prefetch = g_l2_prefetch_tiles.load(std::memory_order_relaxed);
+  p.l2_prefetch = l2_prefetch_setting();
   p.stall_tx = g_stall_tx.load(std::memory_order_relaxed);
   if (rope) rope_turns_table(rope_theta, m.d, p.rope_turns);
   else memset(p.rope_turns, 0, sizeof(p.rope_turns));

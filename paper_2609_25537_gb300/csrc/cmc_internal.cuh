@@ -26,6 +26,9 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+// The setting of cmc_set_l2_prefetch_tiles.
+int l2_prefetch_setting();
+
 // Validates the shape fields of a cmc_dims that the attention path uses.
 int validate_dims(const cmc_dims* dims, bool need_bank);
 

@@ -62,3 +62,24 @@ def test_rejects_unpinned_host_memory(cuda_device):
     with pytest.raises(ValueError, match="pinned"):
         cmc.stage_copies([(torch.zeros(64, dtype=torch.uint8),
                            torch.zeros(64, dtype=torch.uint8, device=cuda_device))])
+
+
+@pytest.mark.parametrize("tiles", [0, 5])
+@pytest.mark.parametrize("nbytes", [16384, 32768, 1 << 20])
+def test_copies_precede_the_next_launch_at_any_prefetch_depth(cuda_device, tiles, nbytes):
+    """The launch after a staging copy sees its bytes whether it may start with the copy (a
+    prefetch depth above 0, or small copies) or with its end."""
+    s = torch.cuda.current_stream(cuda_device)
+    src = [_bytes(nbytes, 10 + i).pin_memory() for i in range(4)]
+    mid = torch.zeros(nbytes, dtype=torch.uint8, device=cuda_device)
+    back = [torch.zeros(nbytes, dtype=torch.uint8).pin_memory() for _ in src]
+    cmc.set_l2_prefetch_tiles(tiles)
+    try:
+        for a, b in zip(src, back):
+            cmc.stage_copies([(a, mid)], wait_first=True)   # after the copy out of mid before it
+            cmc.stage_copies([(mid, b)], wait_first=True)
+        s.synchronize()
+    finally:
+        cmc.set_l2_prefetch_tiles(5)
+    for a, b in zip(src, back):
+        assert torch.equal(a, b)
